@@ -1,0 +1,13 @@
+// pa_eval_lanes_asy2.cu -- the lane-per-chromosome FP32 evaluation
+// (pa_eval_lanes.cuh), asymptotic SINR, float2 table rows: a translation unit of its
+// own so that the variants compile in parallel.
+#include "pa_eval_lanes.cuh"
+
+namespace pa {
+
+cudaError_t lanes_dispatch_asy2(int NC, const LanesArgs& a, size_t smem, int num_sms,
+                                int64_t tiles, cudaStream_t st) {
+  return pick_lanes<2, false>(NC, a, smem, num_sms, tiles, st);
+}
+
+}  // namespace pa

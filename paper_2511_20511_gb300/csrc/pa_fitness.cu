@@ -372,6 +372,8 @@ F32Launch f32_shape(int L, int K, int RS, int NJ) {
   return s;
 }
 
+}  // namespace
+
 // Resident blocks per SM of a kernel at a launch shape.  The first query of
 // a kernel on a device raises its dynamic shared-memory cap to the device's
 // opt-in maximum (a cap sized to one launch would reject a later, larger
@@ -382,7 +384,7 @@ struct OccKey {
   int dev, threads;
   size_t smem;
 };
-static int cached_occupancy(const void* fn, int threads, size_t smem, cudaError_t* err) {
+int cached_occupancy(const void* fn, int threads, size_t smem, cudaError_t* err) {
   static OccKey keys[256];
   static int vals[256];
   static int used = 0;
@@ -419,6 +421,8 @@ static int cached_occupancy(const void* fn, int threads, size_t smem, cudaError_
   }
   return per_sm;
 }
+
+namespace {
 
 template <int NJ, int VEC, bool FIN>
 cudaError_t run_f32(const F32Args& a, const F32Launch& s, int num_sms, cudaStream_t st) {
@@ -528,6 +532,8 @@ cudaError_t launch_eval_f32(pa_ctx* ctx, const uint8_t* pop, int64_t n, float* f
                             cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
   const pa::F32Tables& t = ctx->t32;
+  const cudaError_t el = launch_eval_lanes(ctx, pop, n, fit, st);
+  if (el != cudaErrorNotSupported) return el;
   const int L = ctx->cfg.L, K = ctx->cfg.K;
   const bool fin = ctx->cfg.mode == PA_SINR_FINITE_M;
   if (pilot_kernel_applies(t.NJ, t.vec, K)) {

@@ -120,6 +120,10 @@ cudaError_t launch_eval_f32(pa_ctx* ctx, const uint8_t* pop, int64_t n, float* f
 cudaError_t launch_eval_f64(const pa_ctx* ctx, const uint8_t* pop, int64_t n, double* fit,
                             cudaStream_t st);
 bool f32_supported(int L, int K, size_t* smem_bytes);
+// pa_eval_lanes.cu: throughput form (a lane per chromosome);
+// cudaErrorNotSupported where it does not apply
+cudaError_t launch_eval_lanes(pa_ctx* ctx, const uint8_t* pop, int64_t n, float* out,
+                              cudaStream_t st);
 // pa_stream.cu: column-tiled evaluation for tables beyond shared memory
 bool f32_stream_geometry(int L, int K, int* JT, int* RSt, int* vec, int* ntile);
 cudaError_t launch_eval_f32_stream(pa_ctx* ctx, const uint8_t* pop, int64_t n, float* fit,

@@ -185,6 +185,17 @@ cudaError_t launch_eval_f32_stream(pa_ctx* ctx, const uint8_t* pop, int64_t n, f
     if (e != cudaSuccess) return e;
     t.partial_cap = n;
   }
+  auto reduce = [&]() {
+    const int64_t rb = std::min<int64_t>((n + 255) / 256, (int64_t)ctx->num_sms * 8);
+    (void)cudaGetLastError();
+    k_stream_reduce<<<(unsigned)rb, 256, 0, st>>>(t.partial, t.ntile, n, fit,
+                                                  ctx->cfg.objective);
+    count_launch();
+    return cudaGetLastError();
+  };
+  cudaError_t e = launch_eval_lanes(ctx, pop, n, t.partial, st);
+  if (e == cudaSuccess) return reduce();
+  if (e != cudaErrorNotSupported) return e;
   const int L = ctx->cfg.L, K = ctx->cfg.K;
   StreamArgs a;
   a.pop = pop;
@@ -210,7 +221,6 @@ cudaError_t launch_eval_f32_stream(pa_ctx* ctx, const uint8_t* pop, int64_t n, f
   const int per_tile = (int)std::max<int64_t>(1, std::min<int64_t>(mtiles, want));
   const int grid = per_tile * t.ntile;
   const bool fin = ctx->cfg.mode == PA_SINR_FINITE_M;
-  cudaError_t e;
   if (t.vec == 2) {
     switch (t.JT) {
       case 16: e = fin ? run_stream<16, 2, true>(a, smem, grid, st) : run_stream<16, 2, false>(a, smem, grid, st); break;
@@ -225,11 +235,7 @@ cudaError_t launch_eval_f32_stream(pa_ctx* ctx, const uint8_t* pop, int64_t n, f
     }
   }
   if (e != cudaSuccess) return e;
-  const int64_t rb = std::min<int64_t>((n + 255) / 256, (int64_t)ctx->num_sms * 8);
-  (void)cudaGetLastError();
-  k_stream_reduce<<<(unsigned)rb, 256, 0, st>>>(t.partial, t.ntile, n, fit, a.obj);
-  count_launch();
-  return cudaGetLastError();
+  return reduce();
 }
 
 }  // namespace pa
