@@ -14,16 +14,15 @@
 // member and four users, pilots clamped below K); counts are packed 16-bit
 // pairs (one load serves two clusters); a lane takes one member, warps
 // split the users when the members are few (device code in
-// pa_island_kmeans.cuh).  Counts and Q are updated from the members that
-// changed cluster (Q from the values the atomics return).  Initial
+// pa_island_kmeans.cuh).  Counts are updated from the members that changed
+// cluster (Q too in the one-CTA form, from the values the atomics return).  Initial
 // centroids are C distinct members by a partial Fisher-Yates shuffle
 // (Philox tag 4, keyed by the generation); Lloyd passes run until no label
 // changes or the pass limit; an emptied cluster keeps its counts.
-// k_island_kmeans_cl runs it on a cluster of up to eight CTAs when counts
-// and population fit in shared memory (each CTA assigns a slice of the
-// members and replays every CTA's changed members into its own copy of the
-// counts); k_island_kmeans on one CTA otherwise (counts in global memory
-// for large C*L*K*K, rows read from global memory for large N*L*K).
+// k_island_kmeans_cl runs it on a cluster of up to sixteen CTAs when their
+// shares of counts and population fit in shared memory (the users are split
+// over the CTAs); k_island_kmeans on one CTA otherwise (counts in global
+// memory for large C*L*K*K, rows read from global memory for large N*L*K).
 
 // Island lists (k_island_lists): members grouped by island in ascending
 // index (off, list) and each member's position in its island (pos), by a
@@ -39,6 +38,9 @@
 
 #include <algorithm>
 #include <atomic>
+#include <mutex>
+#include <utility>
+#include <vector>
 
 #include "pa_island_kmeans.cuh"
 
@@ -46,6 +48,7 @@ namespace pa {
 namespace {
 
 constexpr int kIslandThreads = 1024;
+constexpr int kKmClThreads = 512;  // of a cluster K-means CTA (25.0 us; 1024 threads: 28.8)
 
 struct KmArgs {
   const uint8_t* pop;  // [N][LK]
@@ -328,54 +331,46 @@ __global__ void __launch_bounds__(kIslandThreads) k_island_kmeans(const KmArgs a
 }
 
 struct KmClArgs {
-  KmArgs a;
-  int Nr;
-  int o_lab, o_chg, o_gchg;
+  const uint8_t* pop;  // [N][LK]
+  KmParams p;
+  KmClLayout k;
+  int32_t* label;      // [N] out
+  int32_t* passes;     // [1] out
 };
 
 // The cluster K-means from a population in global memory.
-__global__ void __launch_bounds__(kIslandThreads) k_island_kmeans_cl(const KmClArgs ca) {
+__global__ void __launch_bounds__(kKmClThreads) k_island_kmeans_cl(const KmClArgs a) {
   cg::cluster_group cluster = cg::this_cluster();
-  const KmArgs& a = ca.a;
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ KmShared sh;
-  const int N = a.N, K = a.K, LK = a.L * a.K, W = (LK + 3) >> 2, NP = a.NP;
   KmView v;
   v.sh = &sh;
-  v.pw = reinterpret_cast<uint32_t*>(smem + a.o_pw);
-  v.NP = NP;
-  v.cnt = reinterpret_cast<uint32_t*>(smem + a.o_cnt);
-  v.CWp = a.CWp;
-  v.lab = reinterpret_cast<int*>(smem + ca.o_lab);
-  v.perm = v.lab + ((N + 3) & ~3);
-  v.chg = reinterpret_cast<int*>(smem + ca.o_chg);
-  v.gchg = reinterpret_cast<int*>(smem + ca.o_gchg);
-  v.sb = reinterpret_cast<int*>(smem + a.o_sb);
-  v.us = a.us;
-  v.Nr = ca.Nr;
-  const KmParams p{a.N, a.L, a.K, a.C, a.max_iter, a.seed, a.gen};
-  uint32_t* pw = v.pw;
+  v.base = smem;
+  v.k = a.k;
+  const int N = a.p.N, K = a.p.K, LK = a.p.L * K;
   const uint8_t* pop = a.pop;
-  // word w of member n holds the pilots of users 4w .. 4w+3
-  const int passes = km_cluster(v, p, cluster, [&](int warp, int sw, int lane) {
-    for (int n = warp; n < N; n += sw) {
+  auto token = cluster.barrier_arrive();
+  auto stage = [&](uint32_t* pw, int NP, int wb, int nw) {
+    const int st = blockDim.x - 32;
+    for (int t = threadIdx.x; t < N * nw; t += st) {
+      const int n = t / nw, w = t - n * nw;
       const uint8_t* X = pop + (int64_t)n * LK;
-      for (int w = lane; w < W; w += 32) {
-        uint32_t x = 0;
+      uint32_t x = 0;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int u = 4 * w + j;
-          x |= (uint32_t)(u < LK ? min((int)X[u], K - 1) : K - 1) << (8 * j);
-        }
-        pw[w * NP + n] = x;
+      for (int j = 0; j < 4; ++j) {
+        const int u = 4 * (wb + w) + j;
+        x |= (uint32_t)(u < LK ? min((int)X[u], K - 1) : 0) << (8 * j);
       }
+      pw[w * NP + n] = x;
     }
-  });
+  };
+  const int passes = km_cluster(v, a.p, cluster, stage,
+                                [&] { cluster.barrier_wait(std::move(token)); });
   const int R = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
   const int n_lo = N * rank / R, n_hi = N * (rank + 1) / R;  // N * R < 2^31
-  for (int n = n_lo + (int)threadIdx.x; n < n_hi; n += blockDim.x) a.label[n] = v.lab[n];
+  const int* lab = reinterpret_cast<const int*>(smem + a.k.o_lab);
+  for (int n = n_lo + (int)threadIdx.x; n < n_hi; n += blockDim.x) a.label[n] = lab[n];
   if (rank == 0 && threadIdx.x == 0 && a.passes) *a.passes = passes;
-  cluster.sync();  // the other CTAs may still read this CTA's lists
 }
 
 // Members grouped by island.  One CTA: counts, prefix over islands, then
@@ -567,96 +562,86 @@ size_t island_cnt_words(int L, int K, int C) {
   return (size_t)L * K * K * (((C + 1) / 2) | 1);
 }
 
-// Cluster form of the K-means (k_island_kmeans_cl): R = min(8, N/32) CTAs,
-// each holding the whole population and its own counts.
+// Cluster form of the K-means (k_island_kmeans_cl): the largest of 16, 8, 4
+// or 2 CTAs that can be resident, with 16 members and (above 2 CTAs) a word of
+// four users for each; where none of those fits, CTAs without users too.
 // cudaErrorNotSupported when it does not apply (fewer than 64 members, a
-// layout beyond shared memory, a cluster shape that cannot be resident).
+// layout beyond shared memory, no cluster shape resident).
 cudaError_t launch_island_kmeans_cl(const pa_ctx* ctx, const uint8_t* pop, int gen, int32_t* labels,
                                     cudaStream_t st) {
   const pa_config& c = ctx->cfg;
   if (c.N < 64) return cudaErrorNotSupported;
-  const int R = std::min(8, std::max(2, c.N / 32));  // portable cluster sizes
-  const int Nr = (c.N + R - 1) / R;
-  const int groups = (Nr + 31) / 32, W = (c.L * c.K + 3) / 4;
-  int us = std::max(1, std::min({kKmSplits, kIslandThreads / 32 / groups, W}));
-  while (us > 1 && km_cl_layout(c.N, c.L, c.K, c.islands, R, us).total > kKmSmemBudget) --us;
-  const KmClLayout k = km_cl_layout(c.N, c.L, c.K, c.islands, R, us);
-  if (k.total > kKmSmemBudget) return cudaErrorNotSupported;
-  // residency of this shape, once per (device, cluster size, shared memory)
+  // residency of a shape, once per (device, cluster size, shared memory)
   struct Fit {
-    int dev, R;
-    size_t smem;
+    int dev, R, smem;
     bool ok;
   };
-  static Fit fits[64];
-  static std::atomic<int> nfits{0};
+  static std::vector<Fit> fits;
+  static std::mutex mu;
   static std::atomic<uint64_t> capped{0};
   const uint64_t bit = 1ULL << (ctx->device & 63);
   if (!(capped.load() & bit)) {
     cudaError_t e = raise_smem_cap((const void*)k_island_kmeans_cl, ctx->device);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k_island_kmeans_cl, cudaFuncAttributeNonPortableClusterSizeAllowed,
+                               1);
     if (e != cudaSuccess) return e;
     capped.fetch_or(bit);
   }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(R, 1, 1);
-  cfg.blockDim = dim3(kIslandThreads, 1, 1);
-  cfg.dynamicSmemBytes = k.total;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = R;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  int known = -1;
-  const int nf = std::min(nfits.load(), 64);
-  for (int i = 0; i < nf; ++i)
-    if (fits[i].dev == ctx->device && fits[i].R == R && fits[i].smem == k.total)
-      known = fits[i].ok ? 1 : 0;
-  if (known < 0) {
-    int nclusters = 0;
-    const bool ok = cudaOccupancyMaxActiveClusters(&nclusters, k_island_kmeans_cl, &cfg) ==
-                        cudaSuccess && nclusters >= 1;
-    (void)cudaGetLastError();
-    const int i = nfits.fetch_add(1);
-    if (i < 64) fits[i] = Fit{ctx->device, R, k.total, ok};
-    known = ok ? 1 : 0;
+  const int W = (c.L * c.K + 3) / 4;
+  for (int t = 0; t < 8; ++t) {
+    const int R = 16 >> (t & 3);
+    if ((R > 2 && R > W) != (t >= 4) || 16 * R > c.N) continue;
+    const KmClLayout k = km_cl_layout(c.N, c.L, c.K, c.islands, R, kKmClThreads,
+                                      (int)kKmSmemBudget);
+    if ((size_t)k.total > kKmSmemBudget) continue;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(R, 1, 1);
+    cfg.blockDim = dim3(kKmClThreads, 1, 1);
+    cfg.dynamicSmemBytes = k.total;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = R;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    bool ok = false;
+    {
+      std::lock_guard<std::mutex> lock(mu);
+      auto it = std::find_if(fits.begin(), fits.end(), [&](const Fit& f) {
+        return f.dev == ctx->device && f.R == R && f.smem == k.total;
+      });
+      if (it == fits.end()) {
+        int nclusters = 0;
+        ok = cudaOccupancyMaxActiveClusters(&nclusters, k_island_kmeans_cl, &cfg) ==
+                 cudaSuccess && nclusters >= 1;
+        (void)cudaGetLastError();
+        if (fits.size() < 256) fits.push_back(Fit{ctx->device, R, k.total, ok});
+      } else {
+        ok = it->ok;
+      }
+    }
+    if (!ok) continue;
+    KmClArgs a;
+    a.pop = pop;
+    a.p = KmParams{c.N, c.L, c.K, c.islands, c.island_iter, c.seed, gen};
+    a.k = k;
+    a.label = labels;
+    a.passes = ctx->isl_passes;
+    (void)cudaGetLastError();  // drop a stale error of an earlier call
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_island_kmeans_cl, a);
+    count_launch();
+    return e;
   }
-  if (!known) return cudaErrorNotSupported;
-  KmClArgs ca;
-  KmArgs& a = ca.a;
-  a.pop = pop;
-  a.N = c.N;
-  a.L = c.L;
-  a.K = c.K;
-  a.C = c.islands;
-  a.max_iter = c.island_iter;
-  a.seed = c.seed;
-  a.gen = gen;
-  a.label = labels;
-  a.cnt_g = nullptr;
-  a.passes = ctx->isl_passes;
-  a.us = us;
-  a.CWp = ((c.islands + 1) / 2) | 1;
-  a.NP = k.NP;
-  a.o_cnt = (int)k.o_cnt;
-  a.o_sb = (int)k.o_sb;
-  a.o_pw = (int)k.o_pw;
-  ca.Nr = k.Nr;
-  ca.o_lab = (int)k.o_lab;
-  ca.o_chg = (int)k.o_chg;
-  ca.o_gchg = (int)k.o_gchg;
-  (void)cudaGetLastError();  // drop a stale error of an earlier call
-  cudaError_t e = cudaLaunchKernelEx(&cfg, k_island_kmeans_cl, ca);
-  count_launch();
-  return e;
+  return cudaErrorNotSupported;
 }
 
 cudaError_t launch_island_kmeans(const pa_ctx* ctx, const uint8_t* pop, int gen, int32_t* labels,
                                  cudaStream_t st) {
   const pa_config& c = ctx->cfg;
-  if (ctx->isl_cnt == nullptr) {  // the cluster form, where it fits and can be resident
+  {  // the cluster form, where it fits and can be resident
     cudaError_t e = launch_island_kmeans_cl(ctx, pop, gen, labels, st);
     if (e != cudaErrorNotSupported) return e;
   }

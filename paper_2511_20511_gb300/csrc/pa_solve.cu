@@ -53,37 +53,17 @@ cudaError_t launch_solve(pa_ctx* ctx, const uint8_t* pop_in, uint8_t* pop_out, i
     SolveShape s = solve_shape(ctx, C, kSoloMaxNP, kSolveThreads);
     if (s.smem > (size_t)kSmemBudget - 64 * 4) continue;
     SolveArgs a{};
-    if (isl_km) {  // K-means arrays after the solve's (KmView of pa_island_kmeans.cuh)
-      const size_t N4 = (size_t)((c.N + 3) & ~3), LK = (size_t)c.L * c.K;
-      const int W = (int)((LK + 3) / 4), NP = c.N | 1, CWp = ((c.islands + 1) / 2) | 1;
-      const int Nr = (c.N + C - 1) / C, groups = (Nr + 31) / 32;
+    if (isl_km) {  // the K-means arrays after the solve's
       auto r16 = [](size_t v) { return (v + 15) & ~size_t(15); };
-      bool fits = false;
-      for (int us = std::max(1, std::min({kKmSplits, kSolveThreads / 32 / groups, W})); us >= 1;
-           --us) {
-        size_t b = r16(s.smem);
-        a.o_ksh = (int)b;
-        b = r16(b + sizeof(KmShared));
-        a.o_kpw = (int)b;
-        b = r16(b + 4 * (size_t)W * NP);
-        a.o_kcnt = (int)b;
-        b = r16(b + 4 * LK * c.K * CWp);
-        a.o_klab = (int)b;
-        b += 4 * 2 * N4;  // labels, initial permutation
-        a.o_kchg = (int)b;
-        b += 4 * 2 * N4;
-        a.o_kgchg = (int)b;
-        b += 4 * N4;
-        a.o_ksb = (int)b;
-        if (us > 1) b += 4 * (size_t)us * c.islands * Nr;
-        a.isl_us = us;
-        if (r16(b) <= (size_t)kSmemBudget - 64 * 4) {
-          s.smem = r16(b);
-          fits = true;
-          break;
-        }
-      }
-      if (!fits) continue;  // no room beside the solve at this cluster size
+      size_t b = r16(s.smem);
+      a.o_ksh = (int)b;
+      b = r16(b + sizeof(KmShared));
+      a.o_km = (int)b;
+      a.km = km_cl_layout(c.N, c.L, c.K, c.islands, C, kSolveThreads,
+                          kSmemBudget - 64 * 4 - (int)b);
+      b += (size_t)a.km.total;
+      if (b > (size_t)kSmemBudget - 64 * 4) continue;  // no room beside the solve at this size
+      s.smem = b;
     }
     a.pop_in = pop_in;
     a.pop_out = pop_out;

@@ -60,11 +60,12 @@ struct SolveArgs {
   int isl_C;
   // re-clustering inside the launch (isl_km): K-means of the population at
   // every generation whose counter is a multiple of isl_R, and at the first
-  // when isl_fresh (at most isl_iter passes, isl_us user splits; shared
-  // memory at the o_k* offsets); the final labels and member lists are
-  // written back to isl_label_out, isl_off_out, isl_list_out, isl_pos_out
-  int isl_km, isl_R, isl_iter, isl_fresh, isl_us;
-  int o_ksh, o_kpw, o_kcnt, o_klab, o_kchg, o_kgchg, o_ksb;
+  // when isl_fresh (at most isl_iter passes; its scalars at o_ksh, its arrays
+  // km at o_km); the final labels and member lists are written back to
+  // isl_label_out, isl_off_out, isl_list_out, isl_pos_out
+  int isl_km, isl_R, isl_iter, isl_fresh;
+  int o_ksh, o_km;
+  KmClLayout km;
   int32_t* isl_label_out;
   int32_t* isl_off_out;
   int32_t* isl_list_out;
@@ -194,16 +195,17 @@ __device__ __forceinline__ int tournament_list(const FT* fit, const int* mem, in
   return best;
 }
 
-// The E best (fitness desc, index asc) of the m members mem[0..m), E <= m,
-// by one warp in E rounds of a warp argmax; out[0..E) by lane 0.
+// The member of rank i (fitness desc, index asc) among the m members
+// mem[0..m), i < min(m, kSmallE), by one warp in i + 1 rounds of a warp argmax.
+// Every lane gets it.
 template <typename FT>
-__device__ __forceinline__ void warp_top_e_list(const FT* fit, const int* mem, int m, int E,
-                                                int lane, int* out) {
-  int chosen[kSmallE];
+__device__ __forceinline__ int warp_rank_list(const FT* fit, const int* mem, int m, int i,
+                                              int lane) {
+  int chosen[kSmallE], last = -1;
 #pragma unroll
   for (int e = 0; e < kSmallE; ++e) {
     chosen[e] = -1;
-    if (e < E) {
+    if (e <= i) {
       int best = -1;
       FT bv = (FT)0;
       for (int t = lane; t < m; t += 32) {
@@ -227,13 +229,10 @@ __device__ __forceinline__ void warp_top_e_list(const FT* fit, const int* mem, i
           bv = ov;
         }
       }
-      chosen[e] = best;
+      chosen[e] = last = best;
     }
   }
-  if (lane == 0)
-#pragma unroll
-    for (int e = 0; e < kSmallE; ++e)
-      if (e < E) out[e] = chosen[e];
+  return last;
 }
 
 // Block-wide best member by (fitness desc, index asc), skipping excluded[0..nex).
@@ -344,46 +343,30 @@ __device__ __forceinline__ void island_recluster(const SolveArgs& a, unsigned ch
                                               cg::cluster_group& cluster,
                                               const unsigned char* popc, int gen, int* ilab,
                                               int* ipos, int* ilist, int* ioff, int* icnt) {
-  const int N = a.N, L = a.L, K = a.K, C = a.isl_C, LK = L * K, NT = a.NT, MS = a.MS;
-  const int W = (LK + 3) >> 2, NP = N | 1, N4 = (N + 3) & ~3;
+  const int N = a.N, L = a.L, K = a.K, C = a.isl_C, NT = a.NT, MS = a.MS;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
-  const int R = (int)cluster.num_blocks();
   KmView kv;
   kv.sh = reinterpret_cast<KmShared*>(smem + a.o_ksh);
-  kv.pw = reinterpret_cast<uint32_t*>(smem + a.o_kpw);
-  kv.NP = NP;
-  kv.cnt = reinterpret_cast<uint32_t*>(smem + a.o_kcnt);
-  kv.CWp = ((C + 1) / 2) | 1;
-  kv.lab = reinterpret_cast<int*>(smem + a.o_klab);
-  kv.perm = kv.lab + N4;
-  kv.chg = reinterpret_cast<int*>(smem + a.o_kchg);
-  kv.gchg = reinterpret_cast<int*>(smem + a.o_kgchg);
-  kv.sb = reinterpret_cast<int*>(smem + a.o_ksb);
-  kv.us = a.isl_us;
-  kv.Nr = (N + R - 1) / R;
+  kv.base = smem + a.o_km;
+  kv.k = a.km;
   const KmParams kp{N, L, K, C, a.isl_iter, a.seed, gen};
-  uint32_t* pw = kv.pw;
   const uint32_t kmask = (uint32_t)(K - 1) * 0x01010101u;
-  km_cluster(kv, kp, cluster, [&](int w0, int sw, int ln) {
-    // pilots of users 4w .. 4w+3 of member n: word w of its record (bytes
-    // past the row are the record's zero padding, never read as users)
+  auto stage = [&](uint32_t* pw, int NP, int wb, int nw) {
+    // words of the members' records (bytes past the row are the record's zero
+    // padding)
     const int nts = (NT & (NT - 1)) == 0 ? __ffs(NT) - 1 : -1;  // owner by a shift
-    for (int n = w0; n < N; n += sw) {
+    const int st = blockDim.x - 32;
+    for (int t = tid; t < N * nw; t += st) {
+      const int w = t / N, n = t - w * N;
       const int r = nts >= 0 ? n >> nts : n / NT;
-      const uint32_t base = dsmem_addr(popc + (n - r * NT) * MS, r);
-      for (int w = ln; w < W; w += 32) pw[w * NP + n] = __vminu4(ld_dsmem(base + 4 * w), kmask);
+      const uint32_t at = dsmem_addr(popc + (n - r * NT) * MS + 4 * (wb + w), r);
+      pw[w * NP + n] = __vminu4(ld_dsmem(at), kmask);
     }
-  });
-  // every CTA's slice is final (written before the last pass's barrier);
-  // member n of CTA r: n < N (r + 1) / R, the smallest such r
-  for (int n = tid; n < N; n += blockDim.x) {
-    int r = (n * R) / N;  // N * R < 2^31
-    while (n >= N * (r + 1) / R) ++r;
-    ilab[n] = *cluster.map_shared_rank(kv.lab + n, r);
-  }
-  for (int c = tid; c < C; c += blockDim.x) icnt[c] = 0;
-  __syncthreads();
-  for (int n = tid; n < N; n += blockDim.x) atomicAdd(&icnt[ilab[n]], 1);
+  };
+  km_cluster(kv, kp, cluster, stage, [] {});
+  const int* lab = reinterpret_cast<const int*>(kv.base + kv.k.o_lab);
+  for (int n = tid; n < N; n += blockDim.x) ilab[n] = lab[n];
+  for (int c = tid; c < C; c += blockDim.x) icnt[c] = kv.sh->nm[c];
   __syncthreads();
   if (tid == 0) {
     int acc = 0;
@@ -459,14 +442,14 @@ __device__ __forceinline__ void solve_body(const SolveArgs& a, unsigned char* sm
   FT* CV = reinterpret_cast<FT*>(p);
   int* CI = reinterpret_cast<int*>(p + sizeof(FT) * 32 * 64);
   // island mode (E <= kSmallE, so the candidates above are not reserved):
-  // labels, positions, member lists, offsets, each island's elites
+  // labels, positions, member lists, offsets, sizes
   const bool isl = ISL && a.isl_C >= 2;
   const int iC = a.isl_C;
   int* ilab = reinterpret_cast<int*>(p);
   int* ipos = ilab + ((N + 3) & ~3);
   int* ilist = ipos + ((N + 3) & ~3);
   int* ioff = ilist + ((N + 3) & ~3);
-  int* ielite = ioff + ((iC + 4) & ~3);  // [C][kSmallE]
+  int* icnt = ioff + ((iC + 4) & ~3);  // [C]
 
   const int base_n = rank * NT;
   const int nvalid = max(0, min(NT, N - base_n));
@@ -578,7 +561,7 @@ __device__ __forceinline__ void solve_body(const SolveArgs& a, unsigned char* sm
     cluster.sync();
     if (g == a.G) break;
     if (ISL && a.isl_km && ((g == 0 && a.isl_fresh) || (a.gen0 + g) % a.isl_R == 0))
-      island_recluster(a, smem, cluster, POPp(cur), a.gen0 + g, ilab, ipos, ilist, ioff, ielite);
+      island_recluster(a, smem, cluster, POPp(cur), a.gen0 + g, ilab, ipos, ilist, ioff, icnt);
     const bool small_e = E <= kSmallE;
     // ---- 3. elites (CTA holding slots below E).  For E <= 8 warp 0 alone
     //         finds them (register lists) and then fills the elite slots while
@@ -649,14 +632,6 @@ __device__ __forceinline__ void solve_body(const SolveArgs& a, unsigned char* sm
       }
       __syncthreads();
     }
-    if (isl) {
-      // each island's min(E, m_c) best members, a warp per island
-      for (int c = warp; c < iC; c += nwarps) {
-        const int m = ioff[c + 1] - ioff[c];
-        warp_top_e_list<FT>(fit, ilist + ioff[c], m, min(E, m), lane, ielite + c * kSmallE);
-      }
-      __syncthreads();
-    }
     if (n_elite_here > 0 && small_e && warp == 0) {
       if (E <= 2)
         warp_top_e_rounds<FT, 2, 8>(fit, N, E, lane, elites);
@@ -696,11 +671,13 @@ __device__ __forceinline__ void solve_body(const SolveArgs& a, unsigned char* sm
         bool elite = false;
         if (isl) {
           // slot n belongs to island c at position i: the island's rank-i
-          // member for i < min(E, m_c), else a child of two tournaments
-          // among the island's members
+          // member for i < min(E, m_c), found by this slot's warp while the
+          // others build their children (a search of all islands before the
+          // children took 1.8 us of a 256-member generation's 7.3), else a
+          // child of two tournaments among the island's members
           const int c = ilab[n], i = ipos[n], m = ioff[c + 1] - ioff[c];
           if (i < min(E, m)) {
-            pa_ = pb_ = ielite[c * kSmallE + i];
+            pa_ = pb_ = warp_rank_list<FT>(fit, ilist + ioff[c], m, i, lane);
             split = LK;
             elite = true;
           } else {
@@ -869,9 +846,9 @@ SolveShape solve_shape(const pa_ctx* ctx, int C, int maxnp, int threads) {
   b = (b + 15) & ~size_t(15);
   b += (size_t)s.CH * s.nblk * 32;
   if (c.E > kSmallE) b += (f64 ? 8 : 4) * 32 * 64 + 4 * 32 * 64;  // elite candidates
-  if (c.islands >= 2) {  // labels, positions, lists, offsets, island elites
+  if (c.islands >= 2) {  // labels, positions, lists, offsets, sizes
     const size_t N4 = (size_t)((c.N + 3) & ~3);
-    b += 4 * (3 * N4 + (size_t)((c.islands + 4) & ~3) + (size_t)c.islands * kSmallE);
+    b += 4 * (3 * N4 + (size_t)((c.islands + 4) & ~3) + (size_t)c.islands);
   }
   s.smem = (b + 15) & ~size_t(15);
   return s;
