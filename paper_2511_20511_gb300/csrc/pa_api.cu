@@ -203,6 +203,7 @@ static void free_ctx(pa_ctx* c) {
   if (!c) return;
   cudaFree(c->arena);
   cudaFree(c->t32.partial);
+  cudaFree(c->t32.inv);
   cudaFreeHost(c->h_best);
   cudaFree(c->stage_pop);
   cudaFree(c->stage_fit);

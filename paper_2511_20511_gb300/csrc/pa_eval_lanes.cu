@@ -15,6 +15,7 @@ namespace pa {
 //   7 x 16   n = 8192: 8.3 / 9.0 us    16384: 11.3 / 10.3   65536: 26.8 / 19.6
 //   37 x 13  n = 1024: 12.4 / 20.6 us   4096: 25.8 / 20.7   65536: 240 / 162
 //   61 x 16 (column tiles)  n = 1024: 22.7 / 24.7 us   4096: 62.0 / 55.7
+//   61 x 32 (column tiles, chunks)  n = 2^17: 2,853 / 2,348 us
 // so the line lies where most SMs get a tile of 32 and the call gathers 12
 // million table words.  Resident tables write fit[n]; column-tiled ones
 // partial[n][ntile].
@@ -26,6 +27,10 @@ cudaError_t launch_eval_lanes(pa_ctx* ctx, const uint8_t* pop, int64_t n, float*
   if (n * ((int64_t)LK * L) < kLanesMinWords) return cudaErrorNotSupported;
   if (t.streamed ? tiles * t.ntile < ctx->num_sms : 5 * tiles < 4 * ctx->num_sms)
     return cudaErrorNotSupported;
+  if (t.streamed) {  // K > 16: chunks of cells
+    const cudaError_t e = launch_eval_chunk(ctx, pop, n, out, st);
+    if (e != cudaErrorNotSupported) return e;
+  }
   LanesArgs a{};
   int cols;  // columns a block holds
   if (t.streamed) {

@@ -81,6 +81,10 @@ using LanesDispatch = cudaError_t(int NC, const LanesArgs& a, size_t smem, int n
                                   int64_t tiles, cudaStream_t st);
 LanesDispatch lanes_dispatch_fin2, lanes_dispatch_fin1, lanes_dispatch_asy2, lanes_dispatch_asy1;
 
+// Column-tiled tables with K > 16 (pa_eval_chunk.cu).
+cudaError_t launch_eval_chunk(pa_ctx* ctx, const uint8_t* pop, int64_t n, float* partial,
+                              cudaStream_t st);
+
 // Resident blocks per SM of a kernel at a launch shape, cached (pa_fitness.cu).
 int cached_occupancy(const void* fn, int threads, size_t smem, cudaError_t* err);
 
@@ -107,43 +111,47 @@ __device__ __forceinline__ void sts8(uint32_t addr, uint32_t v) {
   asm volatile("st.shared.u8 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
 
+// Users k .. k+3 (the first n of them real) of four rows, a word each: byte b
+// of v[s] is the pilot of user k + b in row s; dst: shared address of lane c's
+// byte of the quad's word for pilot 0.  A valid row's bytes are below K: one
+// test for all sixteen (bytes with the top bit set, or reaching it when 128 - K
+// is added), byte by byte otherwise.  dp4a with one non-zero selector byte is a
+// byte's extraction, scaling by the 128 bytes between pilots and base addition
+// in one instruction.
+__device__ __forceinline__ void lanes_put(uint32_t (&v)[4], uint32_t dst, uint32_t k, int n,
+                                          int K) {
+  const uint32_t lim = (uint32_t)(128 - K) * 0x01010101u;
+  if (n < 4) {
+    const uint32_t keep = (1u << (8 * n)) - 1u;
+#pragma unroll
+    for (int s = 0; s < 4; ++s) v[s] &= keep;
+  }
+  uint32_t odd = 0;
+#pragma unroll
+  for (int s = 0; s < 4; ++s) odd |= v[s] | (v[s] + lim);
+  if ((odd & 0x80808080u) == 0) {
+#pragma unroll
+    for (int b = 0; b < 4; ++b)
+      if (b < n) {
+#pragma unroll
+        for (int s = 0; s < 4; ++s) sts8(__dp4a(v[s], 128u << (8 * b), dst) + s, k + b);
+      }
+  } else {
+    for (int b = 0; b < 4 && b < n; ++b)
+#pragma unroll
+      for (int s = 0; s < 4; ++s) {
+        const uint32_t p = (v[s] >> (8 * b)) & 0xffu;
+        if (p < (uint32_t)K) sts8(dst + p * 128 + s, k + b);
+      }
+  }
+}
+
 // Sixteen users k0 .. k0+15 (the first nb of them real) of four rows K bytes
-// apart, row: shared address of user k0's byte of the first; dst: shared
-// address of lane c's byte of the quad's word for pilot 0.  dp4a with one
-// non-zero selector byte is a byte's extraction, scaling by the 128 bytes
-// between pilots and base addition in one instruction.
+// apart, row: shared address of user k0's byte of the first.
 __device__ __forceinline__ void lanes_decode16(uint32_t row, uint32_t dst, int k0, int nb, int K) {
   constexpr int R = 4;
-  // a valid row's bytes are below K: one test for four users of the rows
-  // (bytes with the top bit set, or reaching it when 128 - K is added), byte
-  // by byte otherwise
-  const uint32_t lim = (uint32_t)(128 - K) * 0x01010101u;
   auto put = [&](uint32_t (&v)[R], int w) {
-    const int n = nb - 4 * w;
-    if (n < 4) {
-      const uint32_t keep = (1u << (8 * n)) - 1u;
-#pragma unroll
-      for (int s = 0; s < R; ++s) v[s] &= keep;
-    }
-    uint32_t odd = 0;
-#pragma unroll
-    for (int s = 0; s < R; ++s) odd |= v[s] | (v[s] + lim);
-    const uint32_t k = (uint32_t)(k0 + 4 * w);
-    if ((odd & 0x80808080u) == 0) {
-#pragma unroll
-      for (int b = 0; b < 4; ++b)
-        if (b < n) {
-#pragma unroll
-          for (int s = 0; s < R; ++s) sts8(__dp4a(v[s], 128u << (8 * b), dst) + s, k + b);
-        }
-    } else {
-      for (int b = 0; b < 4 && b < n; ++b)
-#pragma unroll
-        for (int s = 0; s < R; ++s) {
-          const uint32_t p = (v[s] >> (8 * b)) & 0xffu;
-          if (p < (uint32_t)K) sts8(dst + p * 128 + s, k + b);
-        }
-    }
+    lanes_put(v, dst, (uint32_t)(k0 + 4 * w), nb - 4 * w, K);
   };
   if (K % 8 == 0) {  // 8-byte rows: L*K/8 odd keeps a half-warp's loads apart
 #pragma unroll

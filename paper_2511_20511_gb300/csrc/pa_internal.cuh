@@ -44,6 +44,8 @@ struct F32Tables {
   int64_t tile_floats = 0;
   float* partial = nullptr;  // scratch: per-(member, tile) fitness partials
   int64_t partial_cap = 0;   // members it can hold
+  uint32_t* inv = nullptr;   // scratch: decoded inverses (pa_eval_chunk.cu)
+  int64_t inv_cap = 0;       // tiles of 32 members it can hold
   int* err_flag = nullptr;   // set by a kernel whose bounded wait gave up
 };
 

@@ -2,8 +2,9 @@
 against the kernels that small calls take, bit for bit, and against the
 oracle: the same population evaluated in one large call and in small chunks.
 Shapes at the edges of its column shares (12, 13, 24, 25, 48 columns), of the
-load widths (K = 16, 17), of the row alignments the decoder tells apart, and
-column-tiled tables; ragged counts; populations off 16-byte alignment."""
+load widths (K = 16, 17), of the row alignments the decoders tell apart, and
+column-tiled tables (16, 8 and 4 columns; whole inverses and chunks of cells);
+ragged counts; populations off 16-byte alignment."""
 import numpy as np
 import pytest
 
@@ -27,6 +28,11 @@ def B():
 
 
 def _instance(L, K):
+    if L > 61:  # beyond the layouts: log-normal gains
+        rng = np.random.default_rng(L * 64 + K)
+        b = np.exp(rng.normal(-20.0, 2.0, size=(L, L, K)))
+        b[np.arange(L), np.arange(L)] *= 50.0
+        return b.astype(np.float32).astype(np.float64)
     full = next(r for r in (7, 19, 37, 61) if r >= L)
     inst = inputs.instance(full, K, seed=L * 64 + K, dtype=np.float32)
     return np.ascontiguousarray(inst["beta"][:L, :L])
@@ -49,7 +55,8 @@ def _chunks(B, ctx, pop, step):
 
 @pytest.mark.parametrize("L,K", [(2, 2), (7, 4), (12, 16), (13, 7), (19, 10), (19, 16), (24, 5),
                                  (25, 16), (37, 13), (37, 16), (48, 3), (19, 17), (13, 32), (7, 40),
-                                 (33, 20), (61, 12), (53, 20), (49, 9)])
+                                 (33, 20), (61, 12), (53, 20), (49, 9), (61, 32), (49, 17),
+                                 (61, 56), (150, 27), (120, 32)])
 @pytest.mark.parametrize("mode,obj", [(1, 0), (0, 0), (1, 1)])
 def test_large_call_equals_small_calls(B, oracle, L, K, mode, obj):
     beta = _instance(L, K)
