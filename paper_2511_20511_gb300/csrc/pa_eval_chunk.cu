@@ -128,10 +128,13 @@ __global__ void __launch_bounds__(kDecodeThreads) k_eval_decode(const uint8_t* _
 }
 
 // JT: columns of a tile; PPW: pilots per warp.  a.n chromosomes, whose inverses
-// are at invg; a.fit: partial[n][ntile].
+// are at invg; a.fit: partial[n][ntile].  With tickets (one per tile of
+// chromosomes, all zero between launches) the block that finishes a tile last
+// adds its column tiles' partials in tile order into fit.
 template <int JT, int PPW, bool FIN>
 __global__ void __launch_bounds__(kChunkThreads, 1)
-    k_eval_f32_chunk(const LanesArgs a, const uint32_t* __restrict__ invg) {
+    k_eval_f32_chunk(const LanesArgs a, const uint32_t* __restrict__ invg, float* __restrict__ fit,
+                     int* __restrict__ tickets) {
   extern __shared__ __align__(128) unsigned char smem[];
   // [0] the table's bulk copies; from 1: a buffer's chunk has landed; from
   // 1 + kChunkBufs: all warps have gathered it
@@ -213,6 +216,23 @@ __global__ void __launch_bounds__(kChunkThreads, 1)
       for (int k = 0; k < w; ++k) v[k] = pair_add(v[k], v[k + w], mo);
     const int64_t n = tile * kLanesTile + lane;
     if (n < a.n) a.fit[n * a.ntile + t] = v[0];
+    if (!tickets) return;
+    __threadfence();  // the partials before the ticket
+    __syncwarp();
+    int done = 0;
+    if (lane == 0) done = atomicAdd(tickets + tile, 1) + 1;
+    done = __shfl_sync(0xffffffffu, done, 0);
+    if (done < a.ntile) return;
+    __threadfence();  // the tickets before the others' partials
+    if (n < a.n) {
+      float s = mo ? __int_as_float(0x7f800000) : 0.f;
+      for (int k = 0; k < a.ntile; ++k) {
+        const float x = __ldcg(a.fit + n * a.ntile + k);
+        s = mo ? fminf(s, x) : s + x;
+      }
+      fit[n] = s;
+    }
+    if (lane == 0) tickets[tile] = 0;
   };
   int64_t q = 0;  // chunks gathered
   int i = 0;      // tiles done
@@ -325,8 +345,8 @@ __global__ void __launch_bounds__(kChunkThreads, 1)
 }
 
 template <int JT, int PPW>
-cudaError_t run_chunk(const LanesArgs& a, const uint32_t* invg, bool fin, size_t smem,
-                      int num_sms, cudaStream_t st) {
+cudaError_t run_chunk(const LanesArgs& a, const F32Tables& t, float* fit, int* tickets, bool fin,
+                      size_t smem, int num_sms, cudaStream_t st) {
   const void* fn = fin ? (const void*)k_eval_f32_chunk<JT, PPW, true>
                        : (const void*)k_eval_f32_chunk<JT, PPW, false>;
   cudaError_t e = cudaSuccess;
@@ -339,24 +359,28 @@ cudaError_t run_chunk(const LanesArgs& a, const uint32_t* invg, bool fin, size_t
   const unsigned grid = (unsigned)(std::min(tiles, want) * a.ntile);
   (void)cudaGetLastError();  // drop a stale error of an earlier call
   if (fin)
-    k_eval_f32_chunk<JT, PPW, true><<<grid, threads, smem, st>>>(a, invg);
+    k_eval_f32_chunk<JT, PPW, true><<<grid, threads, smem, st>>>(a, t.inv, fit, tickets);
   else
-    k_eval_f32_chunk<JT, PPW, false><<<grid, threads, smem, st>>>(a, invg);
+    k_eval_f32_chunk<JT, PPW, false><<<grid, threads, smem, st>>>(a, t.inv, fit, tickets);
   count_launch();
   return cudaGetLastError();
 }
 
 }  // namespace
 
-// Column-tiled tables with K > 16 (scalar rows) into partial[n][ntile].
-// cudaErrorNotSupported for other tables, or where it does not fit (shared
-// memory, or device memory for the inverses of kChunkSlab chromosomes: the
-// context keeps them, at most 256 MB or so).
-cudaError_t launch_eval_chunk(pa_ctx* ctx, const uint8_t* pop, int64_t n, float* partial,
-                              cudaStream_t st) {
+// Column-tiled tables with K > 16 (scalar rows): the fitness of n chromosomes;
+// t.partial holds n * ntile values.  cudaErrorNotSupported for other tables,
+// small calls (lanes_applies), or where it does not fit (shared memory, or
+// device memory for the inverses of kChunkSlab chromosomes: the context keeps
+// them, at most 256 MB or so).  *summed: fit is written, else the caller adds
+// the partials.  Where a block has few tiles, tickets save the launch that adds
+// the partials (4 us of a generation's 78 at n = 2048); with many, the fence
+// behind each tile costs more (2^17: 2,428 us against 2,348).
+cudaError_t launch_eval_chunk(pa_ctx* ctx, const uint8_t* pop, int64_t n, float* fit,
+                              bool* summed, cudaStream_t st) {
   F32Tables& t = ctx->t32;
   const int L = ctx->cfg.L, K = ctx->cfg.K, LK = L * K;
-  if (!t.streamed || t.vec != 1) return cudaErrorNotSupported;
+  if (!t.streamed || t.vec != 1 || !lanes_applies(ctx, n)) return cudaErrorNotSupported;
   const int PPW = K <= kChunkThreads / 32 ? 1 : 2;
   if (t.JT == 16 && PPW != 1) return cudaErrorNotSupported;  // (too many sums per thread)
   LanesArgs a{};
@@ -386,10 +410,14 @@ cudaError_t launch_eval_chunk(pa_ctx* ctx, const uint8_t* pop, int64_t n, float*
     cudaFree(t.inv);
     t.inv = nullptr;
     t.inv_cap = 0;
-    if (cudaMalloc(&t.inv, 4 * (size_t)a.inv_words * nch * slab_tiles) != cudaSuccess) {
+    const size_t inv_bytes = 4 * (size_t)a.inv_words * nch * slab_tiles;
+    if (cudaMalloc(&t.inv, inv_bytes + sizeof(int) * slab_tiles) != cudaSuccess) {
       (void)cudaGetLastError();
       return cudaErrorNotSupported;
     }
+    t.tickets = reinterpret_cast<int*>(reinterpret_cast<unsigned char*>(t.inv) + inv_bytes);
+    const cudaError_t e = cudaMemsetAsync(t.tickets, 0, sizeof(int) * slab_tiles, st);
+    if (e != cudaSuccess) return e;
     t.inv_cap = slab_tiles;
   }
   a.tab = t.tab;
@@ -402,9 +430,11 @@ cudaError_t launch_eval_chunk(pa_ctx* ctx, const uint8_t* pop, int64_t n, float*
   a.pc = t.pc;
   a.obj = ctx->cfg.objective;
   const bool fin = ctx->cfg.mode == PA_SINR_FINITE_M;
+  *summed = slab_tiles * t.ntile <= 4 * (int64_t)ctx->num_sms;  // (then one slab)
+  int* tickets = *summed ? t.tickets : nullptr;
   for (int64_t n0 = 0; n0 < n; n0 += slab) {
     a.n = std::min(slab, n - n0);
-    a.fit = partial + n0 * t.ntile;
+    a.fit = t.partial + n0 * t.ntile;
     a.stall = ctx->test_stall;
     ctx->test_stall = 0;
     const uint8_t* x = pop + n0 * LK;
@@ -418,11 +448,11 @@ cudaError_t launch_eval_chunk(pa_ctx* ctx, const uint8_t* pop, int64_t n, float*
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     switch (t.JT * 10 + PPW) {
-      case 161: e = run_chunk<16, 1>(a, t.inv, fin, b, ctx->num_sms, st); break;
-      case 81: e = run_chunk<8, 1>(a, t.inv, fin, b, ctx->num_sms, st); break;
-      case 82: e = run_chunk<8, 2>(a, t.inv, fin, b, ctx->num_sms, st); break;
-      case 41: e = run_chunk<4, 1>(a, t.inv, fin, b, ctx->num_sms, st); break;
-      case 42: e = run_chunk<4, 2>(a, t.inv, fin, b, ctx->num_sms, st); break;
+      case 161: e = run_chunk<16, 1>(a, t, fit + n0, tickets, fin, b, ctx->num_sms, st); break;
+      case 81: e = run_chunk<8, 1>(a, t, fit + n0, tickets, fin, b, ctx->num_sms, st); break;
+      case 82: e = run_chunk<8, 2>(a, t, fit + n0, tickets, fin, b, ctx->num_sms, st); break;
+      case 41: e = run_chunk<4, 1>(a, t, fit + n0, tickets, fin, b, ctx->num_sms, st); break;
+      case 42: e = run_chunk<4, 2>(a, t, fit + n0, tickets, fin, b, ctx->num_sms, st); break;
       default: return cudaErrorInvalidValue;
     }
     if (e != cudaSuccess) return e;

@@ -7,30 +7,33 @@
 
 namespace pa {
 
-// cudaErrorNotSupported where the kernel does not apply: its buffers exceed
-// shared memory, or the call is so small that the kernels with fewer
-// chromosomes per block (pa_fitness.cu, pa_stream.cu) spread it over more SMs
-// and start sooner.  Measured on GB300, those kernels against this one:
+// Small calls stay with the kernels of fewer chromosomes per block
+// (pa_fitness.cu, pa_stream.cu), which spread them over more SMs and start
+// sooner.  Measured on GB300, those kernels against these:
 //   19 x 10  n = 1024: 10.3 / 12.4 us   4096: 12.4 / 12.4   65536: 51.8 / 43.3
 //   7 x 16   n = 8192: 8.3 / 9.0 us    16384: 11.3 / 10.3   65536: 26.8 / 19.6
 //   37 x 13  n = 1024: 12.4 / 20.6 us   4096: 25.8 / 20.7   65536: 240 / 162
 //   61 x 16 (column tiles)  n = 1024: 22.7 / 24.7 us   4096: 62.0 / 55.7
 //   61 x 32 (column tiles, chunks)  n = 2^17: 2,853 / 2,348 us
 // so the line lies where most SMs get a tile of 32 and the call gathers 12
-// million table words.  Resident tables write fit[n]; column-tiled ones
-// partial[n][ntile].
+// million table words.
+bool lanes_applies(const pa_ctx* ctx, int64_t n) {
+  const F32Tables& t = ctx->t32;
+  const int64_t L = ctx->cfg.L, LK = L * ctx->cfg.K;
+  const int64_t tiles = (n + kLanesTile - 1) / kLanesTile;
+  if (n * LK * L < kLanesMinWords) return false;
+  return t.streamed ? tiles * t.ntile >= ctx->num_sms : 5 * tiles >= 4 * ctx->num_sms;
+}
+
+// cudaErrorNotSupported where the kernel does not apply: a small call, or its
+// buffers exceed shared memory.  Resident tables write fit[n]; column-tiled
+// ones partial[n][ntile].
 cudaError_t launch_eval_lanes(pa_ctx* ctx, const uint8_t* pop, int64_t n, float* out,
                               cudaStream_t st) {
+  if (!lanes_applies(ctx, n)) return cudaErrorNotSupported;
   const F32Tables& t = ctx->t32;
   const int L = ctx->cfg.L, K = ctx->cfg.K, LK = L * K;
   const int64_t tiles = (n + kLanesTile - 1) / kLanesTile;
-  if (n * ((int64_t)LK * L) < kLanesMinWords) return cudaErrorNotSupported;
-  if (t.streamed ? tiles * t.ntile < ctx->num_sms : 5 * tiles < 4 * ctx->num_sms)
-    return cudaErrorNotSupported;
-  if (t.streamed) {  // K > 16: chunks of cells
-    const cudaError_t e = launch_eval_chunk(ctx, pop, n, out, st);
-    if (e != cudaErrorNotSupported) return e;
-  }
   LanesArgs a{};
   int cols;  // columns a block holds
   if (t.streamed) {

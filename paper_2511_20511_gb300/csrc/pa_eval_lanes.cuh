@@ -81,9 +81,9 @@ using LanesDispatch = cudaError_t(int NC, const LanesArgs& a, size_t smem, int n
                                   int64_t tiles, cudaStream_t st);
 LanesDispatch lanes_dispatch_fin2, lanes_dispatch_fin1, lanes_dispatch_asy2, lanes_dispatch_asy1;
 
-// Column-tiled tables with K > 16 (pa_eval_chunk.cu).
-cudaError_t launch_eval_chunk(pa_ctx* ctx, const uint8_t* pop, int64_t n, float* partial,
-                              cudaStream_t st);
+// Whether a call of n chromosomes is large enough for these kernels
+// (pa_eval_lanes.cu).
+bool lanes_applies(const pa_ctx* ctx, int64_t n);
 
 // Resident blocks per SM of a kernel at a launch shape, cached (pa_fitness.cu).
 int cached_occupancy(const void* fn, int threads, size_t smem, cudaError_t* err);

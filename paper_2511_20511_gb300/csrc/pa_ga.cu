@@ -5,7 +5,7 @@
 // seed and addressed by (slot, generation, tag), so a child's draws do not
 // depend on which thread makes them and the generation is bit-reproducible.
 //
-// GA generation (one thread per child slot n):
+// GA generation (one warp per child slot n):
 //   slots 0..E-1  the E best members by (fitness desc, index asc), unchanged
 //                 (elitism);
 //   slot n >= E   parent a = tournament over draws [0, t), parent b over
@@ -102,77 +102,201 @@ struct GaArgs {
   int gen;
 };
 
-// Best of the candidates drawn by draws dr[0 .. T) (indices uniform with
-// replacement), by (fitness desc, index asc): the winner does not depend on
-// the order the candidates are compared in, so lanes split the work.
+constexpr int kGaThreads = 256;
+constexpr int kGaWarps = kGaThreads / 32;
+
+// (value v of member i) better than (bv, b): higher, or not lower and a lower
+// index; b < 0: nothing yet.
 template <typename FT>
-__device__ __forceinline__ int warp_tournament(const FT* fit, int N, int T, const uint32_t* dr,
-                                               int lane) {
-  int best = -1;
-  for (int t = lane; t < T; t += 32) {
-    const int c = (int)below(dr[t], (uint32_t)N);
-    if (best < 0 || better(fit, c, best)) best = c;
-  }
-  for (int off = 16; off > 0; off >>= 1) {
-    const int o = __shfl_xor_sync(0xffffffffu, best, off);
-    if (o >= 0 && (best < 0 || better(fit, o, best))) best = o;
-  }
-  return best;
+__device__ __forceinline__ bool better_val(FT v, int i, FT bv, int b) {
+  if (b < 0) return true;
+  if (v > bv) return true;
+  if (v < bv) return false;
+  return i < b;
 }
 
-constexpr int kGaThreads = 256;
-constexpr int kGaChildren = 8;  // child slots per block (one warp each)
-
-// One block per 8 consecutive child slots.  The block first generates all
-// their draws (one Philox block per thread) into shared memory, then each
-// warp builds one child: tournaments in parallel lanes, the parents' rows
-// copied with coalesced byte streams, the per-row swap mutation with one
-// lane per row.
+// Winner of the candidates (c, v) of the 2^lg lanes around this one (c < 0:
+// none), in each of them.
 template <typename FT>
-__global__ void __launch_bounds__(kGaThreads) k_ga_step(const GaArgs a) {
-  extern __shared__ uint32_t DR[];  // [kGaChildren][nblk*8]
-  __shared__ int elites[64];
-  __shared__ int red[33];
+__device__ __forceinline__ void lanes_best(int& c, FT& v, int width) {
+  for (int off = width >> 1; off > 0; off >>= 1) {
+    const int o = __shfl_xor_sync(0xffffffffu, c, off);
+    const FT ov = __shfl_xor_sync(0xffffffffu, v, off);
+    if (o >= 0 && better_val(ov, o, v, c)) {
+      c = o;
+      v = ov;
+    }
+  }
+}
+
+// The E best members into slots 0 .. E-1, by one block: E rounds of a block
+// argmax over the fitness, of which each thread keeps its first kGaCache values
+// in registers (larger populations re-read the rest); one barrier per round
+// (the warps' results are double-buffered, every thread reduces them).
+constexpr int kGaCache = 8;
+template <typename FT>
+__device__ void ga_elites(const GaArgs& a, int* elites, int* wi, FT* wv) {
   const FT* fit = static_cast<const FT*>(a.fit);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  FT vc[kGaCache];
+  uint32_t taken = 0;
+#pragma unroll
+  for (int r = 0; r < kGaCache; ++r) {
+    const int i = tid + kGaThreads * r;
+    vc[r] = i < a.N ? __ldg(fit + i) : (FT)0;
+  }
+  for (int e = 0; e < a.E; ++e) {
+    int best = -1;
+    FT bv = (FT)0;
+#pragma unroll
+    for (int r = 0; r < kGaCache; ++r) {
+      const int i = tid + kGaThreads * r;
+      if (i < a.N && !(taken >> r & 1) && better_val(vc[r], i, bv, best)) {
+        best = i;
+        bv = vc[r];
+      }
+    }
+    for (int i = tid + kGaThreads * kGaCache; i < a.N; i += kGaThreads) {
+      bool skip = false;
+      for (int f = 0; f < e; ++f) skip |= elites[f] == i;
+      if (skip) continue;
+      const FT v = __ldg(fit + i);
+      if (better_val(v, i, bv, best)) {
+        best = i;
+        bv = v;
+      }
+    }
+    lanes_best(best, bv, 32);
+    const int p = (e & 1) * kGaWarps;
+    if (lane == 0) {
+      wi[p + warp] = best;
+      wv[p + warp] = bv;
+    }
+    __syncthreads();
+    best = -1;
+#pragma unroll
+    for (int w = 0; w < kGaWarps; ++w) {
+      const int o = wi[p + w];
+      const FT ov = wv[p + w];
+      if (o >= 0 && better_val(ov, o, bv, best)) {
+        best = o;
+        bv = ov;
+      }
+    }
+    if (tid == 0) elites[e] = best;  // read after the next barrier
+    if (best % kGaThreads == tid && best / kGaThreads < kGaCache) taken |= 1u << (best / kGaThreads);
+    if (a.N > kGaThreads * kGaCache) __syncthreads();  // the list is read in the next round
+  }
+  __syncthreads();
   const int64_t LK = (int64_t)a.L * a.K;
-  const int E = a.E, T = a.tour;
+  for (int e = warp; e < a.E; e += kGaWarps) {
+    const uint8_t* __restrict__ src = a.pop + (int64_t)elites[e] * LK;
+    uint8_t* __restrict__ dst = a.next + (int64_t)e * LK;
+    for (int64_t i = lane; i < LK; i += 32) dst[i] = src[i];
+  }
+}
+
+// Bytes i .. i+W-1 of a child: from A below split, from B from there on (the
+// unit holding the cut byte by byte).
+template <typename V>
+__device__ __forceinline__ void ga_copy(uint8_t* child, const uint8_t* __restrict__ A,
+                                        const uint8_t* __restrict__ B, int LK, int split,
+                                        int lane) {
+  constexpr int W = (int)sizeof(V);
+#pragma unroll 4
+  for (int i = lane * W; i < LK; i += 32 * W) {
+    if (i + W <= split || i >= split) {
+      const uint8_t* src = i + W <= split ? A : B;
+      *reinterpret_cast<V*>(child + i) = __ldg(reinterpret_cast<const V*>(src + i));
+    } else {
+      for (int j = i; j < i + W; ++j) child[j] = __ldg((j < split ? A : B) + j);
+    }
+  }
+}
+
+// A warp per child, nothing shared between warps: the child's draws (a Philox
+// block per lane) into its shared memory, both tournaments side by side in the
+// two half-warps with the candidates' fitness in registers, the parents' rows
+// copied into shared memory in units of up to 16 bytes, the per-row swaps there
+// (a lane a row), and the child written out.  The last block finds the elites
+// meanwhile.  What bounds it is latency: a chain of one Philox block, a fitness
+// load, a parent load and the stores (61 x 32, N = 2048, cold caches: 17 us; with
+// a block per eight children, the elites searched by the first of them before
+// its children, tournaments re-reading the fitness at each comparison and rows
+// copied bytewise: 25.4 us).
+template <typename FT>
+__global__ void __launch_bounds__(kGaThreads) k_ga_step(const GaArgs a, int width) {
+  extern __shared__ __align__(16) unsigned char gsm[];
+  __shared__ int elites[64];
+  __shared__ int wi[2 * kGaWarps];
+  __shared__ FT wv[2 * kGaWarps];
+  const FT* fit = static_cast<const FT*>(a.fit);
+  const int E = a.E, T = a.tour, LK = a.L * a.K;
+  if (E > 0 && blockIdx.x == gridDim.x - 1) {
+    ga_elites<FT>(a, elites, wi, wv);
+    return;
+  }
   const int nblk = (2 * T + 2 + 3 * a.L + 7) / 8;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int n0 = blockIdx.x * kGaChildren; n0 < a.N; n0 += gridDim.x * kGaChildren) {
-    const int nc = min(kGaChildren, a.N - n0);
-    if (n0 < E) {
-      for (int e = 0; e < E; ++e) {
-        const int b = block_best(fit, a.N, elites, e, red);
-        if (threadIdx.x == 0) elites[e] = b;
-        __syncthreads();
-      }
-    }
-    gen_child_draws(DR, n0, nc, nblk, a.seed, (uint64_t)a.gen, E);
-    __syncthreads();
-    if (warp < nc) {
-      const int n = n0 + warp;
-      uint8_t* __restrict__ child = a.next + n * LK;
-      if (n < E) {
-        const uint8_t* __restrict__ src = a.pop + (int64_t)elites[n] * LK;
-        for (int64_t i = lane; i < LK; i += 32) child[i] = src[i];
-      } else {
-        const uint32_t* dr = DR + (size_t)warp * nblk * 8;
-        const int pa_ = warp_tournament(fit, a.N, T, dr, lane);
-        const int pb_ = warp_tournament(fit, a.N, T, dr + T, lane);
-        int cut = a.L;
-        if ((uint64_t)dr[2 * T] < a.pc_thresh) cut = 1 + (int)below(dr[2 * T + 1], (uint32_t)(a.L - 1));
-        const uint8_t* __restrict__ A = a.pop + (int64_t)pa_ * LK;
-        const uint8_t* __restrict__ B = a.pop + (int64_t)pb_ * LK;
-        const int64_t split = (int64_t)cut * a.K;
-        for (int64_t i = lane; i < LK; i += 32) child[i] = i < split ? A[i] : B[i];
-        __syncwarp();
-        for (int l = lane; l < a.L; l += 32) {
-          const int base = 2 * T + 2 + 3 * l;
-          if ((uint64_t)dr[base] < a.pm_thresh) swap_two(child + (int64_t)l * a.K, a.K, dr[base + 1], dr[base + 2]);
+  const int nw = ((int)gridDim.x - (E > 0 ? 1 : 0)) * kGaWarps;
+  unsigned char* mine = gsm + (size_t)warp * (nblk * 32 + ((LK + 15) & ~15));
+  uint32_t* dr = reinterpret_cast<uint32_t*>(mine);
+  uint8_t* child = mine + nblk * 32;
+  for (int n = E + blockIdx.x * kGaWarps + warp; n < a.N; n += nw) {
+    gen_child_draws_from(dr, n, 1, nblk, a.seed, (uint64_t)a.gen, 0, lane, 32);
+    __syncwarp();
+    int par[2];
+    if (T <= 16) {  // one tournament per half-warp
+      const int h = lane >> 4, t = lane & 15;
+      int c = t < T ? (int)below(dr[h * T + t], (uint32_t)a.N) : -1;
+      FT v = c >= 0 ? __ldg(fit + c) : (FT)0;
+      lanes_best(c, v, 16);
+      par[0] = __shfl_sync(0xffffffffu, c, 0);
+      par[1] = __shfl_sync(0xffffffffu, c, 16);
+    } else {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        int best = -1;
+        FT bv = (FT)0;
+        for (int t = lane; t < T; t += 32) {
+          const int c = (int)below(dr[h * T + t], (uint32_t)a.N);
+          const FT v = __ldg(fit + c);
+          if (better_val(v, c, bv, best)) {
+            best = c;
+            bv = v;
+          }
         }
+        lanes_best(best, bv, 32);
+        par[h] = best;
       }
     }
-    __syncthreads();
+    int cut = a.L;
+    if ((uint64_t)dr[2 * T] < a.pc_thresh) cut = 1 + (int)below(dr[2 * T + 1], (uint32_t)(a.L - 1));
+    const uint8_t* A = a.pop + (int64_t)par[0] * LK;
+    const uint8_t* B = a.pop + (int64_t)par[1] * LK;
+    const int split = cut * a.K;
+    if (width == 16)
+      ga_copy<uint4>(child, A, B, LK, split, lane);
+    else if (width == 4)
+      ga_copy<uint32_t>(child, A, B, LK, split, lane);
+    else
+      ga_copy<uint8_t>(child, A, B, LK, split, lane);
+    __syncwarp();
+    for (int l = lane; l < a.L; l += 32) {
+      const int base = 2 * T + 2 + 3 * l;
+      if ((uint64_t)dr[base] < a.pm_thresh) swap_two(child + l * a.K, a.K, dr[base + 1], dr[base + 2]);
+    }
+    __syncwarp();
+    uint8_t* dst = a.next + (int64_t)n * LK;
+    if (width == 16)
+      for (int i = lane * 16; i < LK; i += 512)
+        *reinterpret_cast<uint4*>(dst + i) = *reinterpret_cast<const uint4*>(child + i);
+    else if (width == 4)
+      for (int i = lane * 4; i < LK; i += 128)
+        *reinterpret_cast<uint32_t*>(dst + i) = *reinterpret_cast<const uint32_t*>(child + i);
+    else
+      for (int i = lane; i < LK; i += 32) dst[i] = child[i];
+    __syncwarp();
   }
 }
 
@@ -530,15 +654,28 @@ cudaError_t launch_ga_step(const pa_ctx* ctx, const uint8_t* pop, const void* fi
   a.pm_thresh = c.pm_thresh;
   a.seed = c.seed;
   a.gen = gen;
-  const int blocks = std::max(1, std::min((c.N + kGaChildren - 1) / kGaChildren,
-                                          ctx->num_sms * 8));
-  const int nblk = (2 * c.tour + 2 + 3 * c.L + 7) / 8;
-  const size_t smem = (size_t)kGaChildren * nblk * 32;
+  const int children = c.N - c.E;
+  const int blocks = std::max(1, std::min((children + kGaWarps - 1) / kGaWarps,
+                                          ctx->num_sms * 8)) + (c.E > 0 ? 1 : 0);
+  const int nblk = (2 * c.tour + 2 + 3 * c.L + 7) / 8, LK = c.L * c.K;
+  const size_t smem = (size_t)kGaWarps * (nblk * 32 + ((LK + 15) & ~15));
+  // units that every member's row starts aligned to, in both buffers
+  const uintptr_t at = reinterpret_cast<uintptr_t>(pop) | reinterpret_cast<uintptr_t>(next);
+  const int width = LK % 16 == 0 && at % 16 == 0 ? 16 : LK % 4 == 0 && at % 4 == 0 ? 4 : 1;
+  const bool f64 = c.prec == PA_FP64;
+  static std::atomic<uint64_t> capped[2];  // devices whose cap is raised (bit per device)
+  const uint64_t bit = 1ULL << (ctx->device & 63);
+  if (smem > 40 * 1024 && !(capped[f64].load() & bit)) {
+    cudaError_t e = raise_smem_cap(f64 ? (const void*)k_ga_step<double>
+                                       : (const void*)k_ga_step<float>, ctx->device);
+    if (e != cudaSuccess) return e;
+    capped[f64].fetch_or(bit);
+  }
   (void)cudaGetLastError();  // drop a stale error of an earlier call
-  if (c.prec == PA_FP64)
-    k_ga_step<double><<<blocks, kGaThreads, smem, st>>>(a);
+  if (f64)
+    k_ga_step<double><<<blocks, kGaThreads, smem, st>>>(a, width);
   else
-    k_ga_step<float><<<blocks, kGaThreads, smem, st>>>(a);
+    k_ga_step<float><<<blocks, kGaThreads, smem, st>>>(a, width);
   count_launch();
   return cudaGetLastError();
 }

@@ -46,6 +46,7 @@ struct F32Tables {
   int64_t partial_cap = 0;   // members it can hold
   uint32_t* inv = nullptr;   // scratch: decoded inverses (pa_eval_chunk.cu)
   int64_t inv_cap = 0;       // tiles of 32 members it can hold
+  int* tickets = nullptr;    // one per such tile, behind inv; zero between launches
   int* err_flag = nullptr;   // set by a kernel whose bounded wait gave up
 };
 
@@ -126,6 +127,10 @@ bool f32_supported(int L, int K, size_t* smem_bytes);
 // cudaErrorNotSupported where it does not apply
 cudaError_t launch_eval_lanes(pa_ctx* ctx, const uint8_t* pop, int64_t n, float* out,
                               cudaStream_t st);
+// pa_eval_chunk.cu: the same for column-tiled tables with K > 16 (t32.partial,
+// and the fitness itself when *summed)
+cudaError_t launch_eval_chunk(pa_ctx* ctx, const uint8_t* pop, int64_t n, float* fit,
+                              bool* summed, cudaStream_t st);
 // pa_stream.cu: column-tiled evaluation for tables beyond shared memory
 bool f32_stream_geometry(int L, int K, int* JT, int* RSt, int* vec, int* ntile);
 cudaError_t launch_eval_f32_stream(pa_ctx* ctx, const uint8_t* pop, int64_t n, float* fit,

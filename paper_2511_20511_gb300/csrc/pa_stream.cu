@@ -193,7 +193,11 @@ cudaError_t launch_eval_f32_stream(pa_ctx* ctx, const uint8_t* pop, int64_t n, f
     count_launch();
     return cudaGetLastError();
   };
-  cudaError_t e = launch_eval_lanes(ctx, pop, n, t.partial, st);
+  bool summed = false;
+  cudaError_t e = launch_eval_chunk(ctx, pop, n, fit, &summed, st);
+  if (e == cudaSuccess) return summed ? e : reduce();
+  if (e != cudaErrorNotSupported) return e;
+  e = launch_eval_lanes(ctx, pop, n, t.partial, st);
   if (e == cudaSuccess) return reduce();
   if (e != cudaErrorNotSupported) return e;
   const int L = ctx->cfg.L, K = ctx->cfg.K;
