@@ -3,6 +3,8 @@
 // pa_fitness.cu and the fused solve kernel of pa_solve.cu.
 #pragma once
 
+#include <type_traits>
+
 #include "pa_internal.cuh"
 
 namespace pa {
@@ -183,6 +185,77 @@ __device__ __forceinline__ float se_pilot_f32(float s2, float s1, float b, float
   return minobj ? __fmul_rn(num, r) : lg2_ftz(__fmaf_rn(num, r, 1.f));
 }
 
+__device__ __forceinline__ uint32_t lds32(uint32_t addr) {
+  uint32_t v;
+  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
+  return v;
+}
+__device__ __forceinline__ uint32_t lds_u8(uint32_t addr) {
+  uint32_t v;
+  asm volatile("ld.shared.u8 %0, [%1];" : "=r"(v) : "r"(addr));
+  return v;
+}
+
+// Packed pairs as 64-bit registers (f32x2 instructions): two independent
+// IEEE single-precision operations, each rounded as the scalar one.
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pk(float x, float y) {
+  f32x2 v;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(x), "f"(y));
+  return v;
+}
+__device__ __forceinline__ float2 upk(f32x2 v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ f32x2 lds_x2(uint32_t addr) {
+  f32x2 v;
+  asm volatile("ld.shared.b64 %0, [%1];" : "=l"(v) : "r"(addr));
+  return v;
+}
+__device__ __forceinline__ float lds_f(uint32_t addr) {
+  float v;
+  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr));
+  return v;
+}
+
+// Values of the two users of one column pair: se_pilot_f32's operations and
+// roundings, two to an instruction where they are packed.
+template <bool FIN, bool MO>
+__device__ __forceinline__ float2 se_pair_f32(f32x2 s2, f32x2 s1, f32x2 b, f32x2 bn, f32x2 M,
+                                              f32x2 pc) {
+  const f32x2 b2 = mul2(b, b);
+  f32x2 num, den;
+  if (FIN) {
+    num = mul2(M, b2);
+    den = fma2(M, s2, mul2(bn, add2(add2(s1, b), pc)));
+  } else {
+    num = b2;
+    den = s2;
+  }
+  const float2 d = upk(den);
+  const f32x2 r = pk(rcp_ftz(d.x), rcp_ftz(d.y));
+  if (MO) return upk(mul2(num, r));
+  const float2 a = upk(fma2(num, r, pk(1.f, 1.f)));
+  return make_float2(lg2_ftz(a.x), lg2_ftz(a.y));
+}
+
 // Combine two users' values of one (pilot, column pair) entry: a sum for the
 // sum-SE objective (starting from 0), a minimum for the max-min objective
 // (starting from +inf, so that padding columns leave the entry unchanged).
@@ -198,15 +271,12 @@ struct PilotSplit {
   static constexpr int JS = (VEC == 2 && NJ >= 8) ? 2 : 1;
 };
 
-// SE of the users holding pilot p in one member, for the BS column pairs
-// [h*NP, (h+1)*NP) with NP = NJ/(2 JS); invp[l*stride] is the user of cell l
-// holding p.  For each cell l the row of user inv_l(p) (its gains at every
-// BS) is added into the accumulators, squared for S2 and plain for S1
-// (FINITE_M).  pair_se[c] receives se(2c) + se(2c+1) for each pair c of the
-// share (zero for columns past L), so that the member's fitness can be
-// summed over (pilot, pair) in one fixed order whatever JS is.
+// The form of eval_pilot_f32 (below; the same values) for one or two pairs per
+// thread, where many threads share a pilot and the shortest code per thread
+// wins (the one-instance solve at 19 x 10: 1,184 us per launch with this form,
+// 1,208 with the other, on one build otherwise).
 template <int NJ, int VEC, bool FIN, int JS>
-__device__ __forceinline__ void eval_pilot_f32(const F32Smem& s, const uint8_t* invp, int stride,
+__device__ __forceinline__ void eval_pilot_short(const F32Smem& s, const uint8_t* invp, int stride,
                                                int h, float* pair_se, bool minobj) {
   static_assert(NJ % (2 * JS) == 0, "NJ must split into JS shares of column pairs");
   constexpr int NP = NJ / 2 / JS;
@@ -252,6 +322,107 @@ __device__ __forceinline__ void eval_pilot_f32(const F32Smem& s, const uint8_t* 
     }
     pair_se[c] = ps;
   }
+}
+
+// SE of the users holding pilot p in one member, for the BS column pairs
+// [h*NP, (h+1)*NP) with NP = NJ/(2 JS); invp[l*stride] is the user of cell l
+// holding p.  For each cell l the row of user inv_l(p) (its gains at every
+// BS) is added into the accumulators, squared for S2 and plain for S1
+// (FINITE_M).  pair_se[c] receives se(2c) + se(2c+1) for each pair c of the
+// share (zero for columns past L), so that the member's fitness can be
+// summed over (pilot, pair) in one fixed order whatever JS is.  Everything is
+// in shared memory; the callers are bound by issue slots as much as by the
+// gathers, so rows are addressed with a constant pitch (a multiply-add and two
+// adds per cell), the users of four cells are fetched ahead of their rows, and
+// the SINR steps work on pairs (se_pair_f32): an evaluation of 128 members of 19 x
+// 10 on one CTA 31,800 -> 29,300 cycles, of 16 of 37 x 16 17,200 -> 16,400.
+template <int NJ, int VEC, bool FIN, int JS>
+__device__ __forceinline__ void eval_pilot_f32(const F32Smem& s, const uint8_t* invp, int stride,
+                                               int h, float* pair_se, bool minobj) {
+  static_assert(NJ % (2 * JS) == 0, "NJ must split into JS shares of column pairs");
+  constexpr int NP = NJ / 2 / JS;
+  if constexpr (NP <= 2) {
+    eval_pilot_short<NJ, VEC, FIN, JS>(s, invp, stride, h, pair_se, minobj);
+    return;
+  }
+  constexpr int RS = VEC == 2 ? NJ + 2 : NJ + 1;  // the table's row pitch
+  f32x2 acc2[NP];
+  f32x2 acc1[FIN ? NP : 1];
+#pragma unroll
+  for (int c = 0; c < NP; ++c) {
+    acc2[c] = 0;
+    if (FIN) acc1[c] = 0;
+  }
+  const int L = s.L, K = s.K;
+  const int c0 = 2 * h * NP;  // first column
+  const uint32_t inv0 = smem_u32(invp), KRS = 4u * K * RS;
+  uint32_t iv = inv0, Tl = smem_u32(s.T) + 4u * c0;
+  auto fetch = [&](uint32_t (&u)[4]) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      u[q] = lds_u8(iv);
+      iv += stride;
+    }
+  };
+  auto cell = [&](uint32_t u) {
+    const uint32_t row = Tl + u * (4u * RS);
+    Tl += KRS;
+#pragma unroll
+    for (int c = 0; c < NP; ++c) {
+      const f32x2 x = VEC == 2 ? lds_x2(row + 8 * c) : pk(lds_f(row + 8 * c), lds_f(row + 8 * c + 4));
+      acc2[c] = fma2(x, x, acc2[c]);
+      if (FIN) acc1[c] = add2(acc1[c], x);
+    }
+  };
+  uint32_t u[4];
+  int l = 0;
+  if (L >= 4) fetch(u);
+  for (; l + 8 <= L; l += 4) {
+    uint32_t un[4];
+    fetch(un);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) cell(u[q]);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) u[q] = un[q];
+  }
+  if (l + 4 <= L) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) cell(u[q]);
+    l += 4;
+  }
+  for (; l < L; ++l) {
+    const uint32_t x = lds_u8(iv);
+    iv += stride;
+    cell(x);
+  }
+  const f32x2 M2 = pk(s.M, s.M), pc2 = pk(s.pc, s.pc);
+  const uint32_t bn = smem_u32(s.BN);
+  auto finish = [&](auto mobj) {
+    constexpr bool mo = decltype(mobj)::value;
+    int j = s.jbase + c0;
+    uint32_t ij = inv0 + j * stride, own = smem_u32(s.OWN) + 4u * j * K;
+#pragma unroll
+    for (int c = 0; c < NP; ++c, j += 2) {
+      float ps = pair_init(mo);
+      if (j < L) {
+        const bool two = j + 1 < L;
+        const float b0 = lds_f(own + 4 * lds_u8(ij));
+        const float b1 = two ? lds_f(own + 4 * K + 4 * lds_u8(ij + stride)) : 1.f;
+        f32x2 bn2 = 0;
+        if (FIN) bn2 = pk(lds_f(bn + 4 * j), two ? lds_f(bn + 4 * j + 4) : 1.f);
+        const float2 x = se_pair_f32<FIN, mo>(acc2[c], FIN ? acc1[c] : 0, pk(b0, b1), bn2, M2, pc2);
+        ps = x.x;
+        if (two) ps = pair_add(ps, x.y, mo);
+      }
+      ij += 2 * stride;
+      own += 8 * K;
+      pair_se[c] = ps;
+    }
+  };
+  if (minobj)
+    finish(std::true_type{});
+  else
+    finish(std::false_type{});
 }
 
 // Fitness of one member from its n per-(pilot, pair) SE sums, by one warp:

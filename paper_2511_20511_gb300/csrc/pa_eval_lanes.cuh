@@ -97,11 +97,6 @@ __device__ __forceinline__ void mbar_arrive(uint32_t mb) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(mb) : "memory");
 }
 
-__device__ __forceinline__ uint32_t lds32(uint32_t addr) {
-  uint32_t v;
-  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
-  return v;
-}
 __device__ __forceinline__ uint2 lds64(uint32_t addr) {
   uint2 v;
   asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(addr));
@@ -204,66 +199,6 @@ __device__ __noinline__ void lanes_decode(uint32_t x, uint32_t inv, int L, int K
     const int nb = min(16, K - k0);
     lanes_decode16(row, dst, k0, nb, K);
   }
-}
-
-// Packed pairs as 64-bit registers (f32x2 instructions): two independent
-// IEEE single-precision operations, each rounded as the scalar one.
-using f32x2 = unsigned long long;
-__device__ __forceinline__ f32x2 pk(float x, float y) {
-  f32x2 v;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(x), "f"(y));
-  return v;
-}
-__device__ __forceinline__ float2 upk(f32x2 v) {
-  float2 r;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-  return r;
-}
-__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
-  f32x2 d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
-__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
-  f32x2 d;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
-  f32x2 d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ f32x2 lds_x2(uint32_t addr) {
-  f32x2 v;
-  asm volatile("ld.shared.b64 %0, [%1];" : "=l"(v) : "r"(addr));
-  return v;
-}
-__device__ __forceinline__ float lds_f(uint32_t addr) {
-  float v;
-  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr));
-  return v;
-}
-
-// Values of the two users of one column pair: se_pilot_f32's operations and
-// roundings, two to an instruction where they are packed.
-template <bool FIN, bool MO>
-__device__ __forceinline__ float2 se_pair_f32(f32x2 s2, f32x2 s1, f32x2 b, f32x2 bn, f32x2 M,
-                                              f32x2 pc) {
-  const f32x2 b2 = mul2(b, b);
-  f32x2 num, den;
-  if (FIN) {
-    num = mul2(M, b2);
-    den = fma2(M, s2, mul2(bn, add2(add2(s1, b), pc)));
-  } else {
-    num = b2;
-    den = s2;
-  }
-  const float2 d = upk(den);
-  const f32x2 r = pk(rcp_ftz(d.x), rcp_ftz(d.y));
-  if (MO) return upk(mul2(num, r));
-  const float2 a = upk(fma2(num, r, pk(1.f, 1.f)));
-  return make_float2(lg2_ftz(a.x), lg2_ftz(a.y));
 }
 
 // Shared addresses a unit reads (lane c's column of the inverse, the tables).

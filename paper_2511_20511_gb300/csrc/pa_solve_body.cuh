@@ -235,6 +235,46 @@ __device__ __forceinline__ int warp_rank_list(const FT* fit, const int* mem, int
   return last;
 }
 
+// The member of rank i (fitness desc, index asc) among the m members
+// mem[0..m), i < min(m, kSmallE), by the sixteen lanes of `mask` (a half-warp)
+// in i + 1 rounds of an argmax.  Each of them gets it.
+template <typename FT>
+__device__ __forceinline__ int half_rank_list(const FT* fit, const int* mem, int m, int i,
+                                              unsigned mask, int hl) {
+  int chosen[kSmallE], last = -1;
+#pragma unroll
+  for (int e = 0; e < kSmallE; ++e) {
+    chosen[e] = -1;
+    if (e <= i) {
+      int best = -1;
+      FT bv = (FT)0;
+      for (int t = hl; t < m; t += 16) {
+        const int c = mem[t];
+        bool taken = false;
+#pragma unroll
+        for (int f = 0; f < e; ++f) taken |= chosen[f] == c;
+        if (taken) continue;
+        const FT v = fit[c];
+        if (best < 0 || better_v(v, c, bv, best)) {
+          best = c;
+          bv = v;
+        }
+      }
+#pragma unroll
+      for (int off = 8; off > 0; off >>= 1) {
+        const int o = __shfl_xor_sync(mask, best, off);
+        const FT ov = __shfl_xor_sync(mask, bv, off);
+        if (o >= 0 && (best < 0 || better_v(ov, o, bv, best))) {
+          best = o;
+          bv = ov;
+        }
+      }
+      chosen[e] = last = best;
+    }
+  }
+  return last;
+}
+
 // Block-wide best member by (fitness desc, index asc), skipping excluded[0..nex).
 template <typename FT>
 __device__ int block_best_s(const FT* fit, int N, const int* excluded, int nex, int* red) {
@@ -405,6 +445,8 @@ __device__ __forceinline__ void solve_body(const SolveArgs& a, unsigned char* sm
   constexpr bool F64 = sizeof(FT) == 8;
   constexpr int JS = F64 ? 1 : fused_js(NJ, MAXNP);
   constexpr int NPR = NJ / 2;  // column pairs per (member, pilot)
+  // the batched column split (many members per CTA) may build two children per warp
+  constexpr bool kHalves = MAXNP != kSoloMaxNP;
 
   // ---- carve shared memory
   unsigned char* p = smem;
@@ -513,9 +555,9 @@ __device__ __forceinline__ void solve_body(const SolveArgs& a, unsigned char* sm
     FT* fit = FITp(g & 1);
     const unsigned char* popc = POPp(cur);
     // ---- 1. evaluate own members, broadcast their fitness.  When all
-    //         children fit in one draw chunk, the threads the evaluation
-    //         leaves idle generate this generation's draws meanwhile (draws
-    //         do not depend on fitness).
+    //         children fit in one draw chunk, this generation's draws are
+    //         generated meanwhile (they do not depend on fitness), by the
+    //         threads the evaluation leaves idle if there are any.
     bool drawn = false;
     for (int c0 = 0; c0 < nvalid; c0 += a.NTT) {
       const int nv = min(a.NTT, nvalid - c0);
@@ -531,7 +573,18 @@ __device__ __forceinline__ void solve_body(const SolveArgs& a, unsigned char* sm
           gen_child_draws_from(DR, base_n, nvalid, nblk, a.seed, (uint64_t)(a.gen0 + g), E_draw,
                                tid - t0, blockDim.x - t0);
         }
-        if (c0 == 0 && one_chunk && eval_threads + 32 <= (int)blockDim.x) drawn = true;
+        if (!kHalves) {
+          if (c0 == 0 && one_chunk && eval_threads + 32 <= (int)blockDim.x) drawn = true;
+        } else if (c0 == 0 && one_chunk) {
+          // no idle threads: every warp draws behind its evaluation, while
+          // others still gather (apart, with a barrier of its own, the draws
+          // took 1,900 of 27,200 cycles at 37 x 16, 8,300 of 59,500 with 128
+          // members of 19 x 10)
+          if (eval_threads + 32 > (int)blockDim.x && g < a.G)
+            gen_child_draws_from(DR, base_n, nvalid, nblk, a.seed, (uint64_t)(a.gen0 + g), E_draw,
+                                 tid, blockDim.x);
+          drawn = true;
+        }
         __syncthreads();
         for (int c = warp; c < nv; c += nwarps) {
           const float f =
@@ -647,100 +700,218 @@ __device__ __forceinline__ void solve_body(const SolveArgs& a, unsigned char* sm
         gen_child_draws(DR, base_n + c0, nc, nblk, a.seed, (uint64_t)(a.gen0 + g), E_draw);
         __syncthreads();
       }
-      // elite slots of a small E are warp 0's (it found the elites); other
-      // slots go round robin to the remaining warps
+      // A warp per child while there are enough warps (the shortest chain),
+      // else a half-warp: a record is 25 16-byte units at 19 x 10 and a
+      // tournament 3 candidates, so that two children share a warp's
+      // instructions (340 per child).  128 members on one CTA: 15,900 -> 12,100
+      // cycles at 19 x 10, 15,400 -> 6,400 at 7 x 8; 16 members on a CTA: a warp
+      // per child 3,000 cycles, halves 4,300.  Elite slots of a small E are warp
+      // 0's (it found the elites); other slots go round robin to the remaining
+      // warps.
       const int ne = (small_e && c0 == 0) ? min(n_elite_here, nc) : 0;
-      const int w_first = ne > 0 ? 1 : 0;
-      const int w_span = nwarps - w_first;
-      int i_begin, i_step;
-      if (ne > 0 && warp == 0) {
-        i_begin = 0;
-        i_step = 1;
-      } else {
-        i_begin = ne + (warp - w_first);
-        i_step = w_span;
-      }
-      const int i_end = (ne > 0 && warp == 0) ? ne : nc;
-      for (int i = i_begin; i < i_end; i += i_step) {
-        const int slot = c0 + i;
-        const int n = base_n + slot;
-        const uint32_t* dr = DR + (size_t)i * nblk * 8;
-        uint32_t* child = reinterpret_cast<uint32_t*>(popn + slot * MS);
-        int pa_, pb_;
-        int64_t split;
-        bool elite = false;
-        if (isl) {
-          // slot n belongs to island c at position i: the island's rank-i
-          // member for i < min(E, m_c), found by this slot's warp while the
-          // others build their children (a search of all islands before the
-          // children took 1.8 us of a 256-member generation's 7.3), else a
-          // child of two tournaments among the island's members
-          const int c = ilab[n], i = ipos[n], m = ioff[c + 1] - ioff[c];
-          if (i < min(E, m)) {
-            pa_ = pb_ = warp_rank_list<FT>(fit, ilist + ioff[c], m, i, lane);
+      if (!kHalves || nc - ne <= nwarps - (ne > 0 ? 1 : 0)) {
+        const int w_first = ne > 0 ? 1 : 0;
+        const int w_span = nwarps - w_first;
+        int i_begin, i_step;
+        if (ne > 0 && warp == 0) {
+          i_begin = 0;
+          i_step = 1;
+        } else {
+          i_begin = ne + (warp - w_first);
+          i_step = w_span;
+        }
+        const int i_end = (ne > 0 && warp == 0) ? ne : nc;
+        for (int i = i_begin; i < i_end; i += i_step) {
+          const int slot = c0 + i;
+          const int n = base_n + slot;
+          const uint32_t* dr = DR + (size_t)i * nblk * 8;
+          uint32_t* child = reinterpret_cast<uint32_t*>(popn + slot * MS);
+          int pa_, pb_;
+          int64_t split;
+          bool elite = false;
+          if (isl) {
+            // slot n belongs to island c at position i: the island's rank-i
+            // member for i < min(E, m_c), found by this slot's warp while the
+            // others build their children (a search of all islands before the
+            // children took 1.8 us of a 256-member generation's 7.3), else a
+            // child of two tournaments among the island's members
+            const int c = ilab[n], i = ipos[n], m = ioff[c + 1] - ioff[c];
+            if (i < min(E, m)) {
+              pa_ = pb_ = warp_rank_list<FT>(fit, ilist + ioff[c], m, i, lane);
+              split = LK;
+              elite = true;
+            } else {
+              pa_ = tournament_list(fit, ilist + ioff[c], m, T_, dr);
+              pb_ = tournament_list(fit, ilist + ioff[c], m, T_, dr + T_);
+              int cut = L;
+              if ((uint64_t)dr[2 * T_] < a.pc_thresh) cut = 1 + (int)below(dr[2 * T_ + 1], (uint32_t)(L - 1));
+              split = (int64_t)cut * K;
+            }
+          } else if (n < E) {
+            pa_ = pb_ = elites[n];
             split = LK;
             elite = true;
           } else {
-            pa_ = tournament_list(fit, ilist + ioff[c], m, T_, dr);
-            pb_ = tournament_list(fit, ilist + ioff[c], m, T_, dr + T_);
+            pa_ = tournament_lane(fit, N, T_, dr);
+            pb_ = tournament_lane(fit, N, T_, dr + T_);
             int cut = L;
             if ((uint64_t)dr[2 * T_] < a.pc_thresh) cut = 1 + (int)below(dr[2 * T_ + 1], (uint32_t)(L - 1));
             split = (int64_t)cut * K;
           }
-        } else if (n < E) {
-          pa_ = pb_ = elites[n];
-          split = LK;
-          elite = true;
-        } else {
-          pa_ = tournament_lane(fit, N, T_, dr);
-          pb_ = tournament_lane(fit, N, T_, dr + T_);
-          int cut = L;
-          if ((uint64_t)dr[2 * T_] < a.pc_thresh) cut = 1 + (int)below(dr[2 * T_ + 1], (uint32_t)(L - 1));
-          split = (int64_t)cut * K;
-        }
-        // parents' records from their owners, 16 bytes per lane and load
-        const int oa = nt_shift >= 0 ? pa_ >> nt_shift : pa_ / NT;
-        const int ob = nt_shift >= 0 ? pb_ >> nt_shift : pb_ / NT;
-        const uint32_t ra = dsmem_addr(POPp(cur) + (pa_ - oa * NT) * MS, oa);
-        const uint32_t rb = dsmem_addr(POPp(cur) + (pb_ - ob * NT) * MS, ob);
-        for (int v = lane; v < (MS >> 4); v += 32) {
-          const uint4 qa = ld_dsmem_v4(ra + 16 * v), qb = ld_dsmem_v4(rb + 16 * v);
-          // bytes below sp from A: the cut in X, and the same cut in INV
-          // (16-byte units never straddle XO); only one unit mixes the two
-          const int lo = 16 * v, sp = lo >= XO ? XO + (int)split : (int)split;
-          uint4 o;
-          if (lo + 16 <= sp) {
-            o = qa;
-          } else if (lo >= sp) {
-            o = qb;
-          } else {
-            o.x = merge_word(qa.x, qb.x, sp - lo);
-            o.y = merge_word(qa.y, qb.y, sp - lo - 4);
-            o.z = merge_word(qa.z, qb.z, sp - lo - 8);
-            o.w = merge_word(qa.w, qb.w, sp - lo - 12);
+          // parents' records from their owners, 16 bytes per lane and load
+          const int oa = nt_shift >= 0 ? pa_ >> nt_shift : pa_ / NT;
+          const int ob = nt_shift >= 0 ? pb_ >> nt_shift : pb_ / NT;
+          const uint32_t ra = dsmem_addr(POPp(cur) + (pa_ - oa * NT) * MS, oa);
+          const uint32_t rb = dsmem_addr(POPp(cur) + (pb_ - ob * NT) * MS, ob);
+          for (int v = lane; v < (MS >> 4); v += 32) {
+            const uint4 qa = ld_dsmem_v4(ra + 16 * v), qb = ld_dsmem_v4(rb + 16 * v);
+            // bytes below sp from A: the cut in X, and the same cut in INV
+            // (16-byte units never straddle XO); only one unit mixes the two
+            const int lo = 16 * v, sp = lo >= XO ? XO + (int)split : (int)split;
+            uint4 o;
+            if (lo + 16 <= sp) {
+              o = qa;
+            } else if (lo >= sp) {
+              o = qb;
+            } else {
+              o.x = merge_word(qa.x, qb.x, sp - lo);
+              o.y = merge_word(qa.y, qb.y, sp - lo - 4);
+              o.z = merge_word(qa.z, qb.z, sp - lo - 8);
+              o.w = merge_word(qa.w, qb.w, sp - lo - 12);
+            }
+            reinterpret_cast<uint4*>(child)[v] = o;
           }
-          reinterpret_cast<uint4*>(child)[v] = o;
-        }
-        __syncwarp();
-        if (!elite) {
-          uint8_t* cx = reinterpret_cast<uint8_t*>(child);
-          for (int l = lane; l < L; l += 32) {
-            const int base = 2 * T_ + 2 + 3 * l;
-            if ((uint64_t)dr[base] < a.pm_thresh && K >= 2) {
-              const int i1 = (int)below(dr[base + 1], (uint32_t)K);
-              const int jj = (int)below(dr[base + 2], (uint32_t)(K - 1));
-              const int i2 = jj + (jj >= i1 ? 1 : 0);
-              uint8_t* xr = cx + l * K;
-              uint8_t* ir = cx + XO + l * K;
-              const uint8_t p1 = xr[i1], p2 = xr[i2];
-              xr[i1] = p2;
-              xr[i2] = p1;
-              if (p1 < K) ir[p1] = (uint8_t)i2;
-              if (p2 < K) ir[p2] = (uint8_t)i1;
+          __syncwarp();
+          if (!elite) {
+            uint8_t* cx = reinterpret_cast<uint8_t*>(child);
+            for (int l = lane; l < L; l += 32) {
+              const int base = 2 * T_ + 2 + 3 * l;
+              if ((uint64_t)dr[base] < a.pm_thresh && K >= 2) {
+                const int i1 = (int)below(dr[base + 1], (uint32_t)K);
+                const int jj = (int)below(dr[base + 2], (uint32_t)(K - 1));
+                const int i2 = jj + (jj >= i1 ? 1 : 0);
+                uint8_t* xr = cx + l * K;
+                uint8_t* ir = cx + XO + l * K;
+                const uint8_t p1 = xr[i1], p2 = xr[i2];
+                xr[i1] = p2;
+                xr[i2] = p1;
+                if (p1 < K) ir[p1] = (uint8_t)i2;
+                if (p2 < K) ir[p2] = (uint8_t)i1;
+              }
             }
           }
+          __syncwarp();
         }
-        __syncwarp();
+      } else {
+        const bool elite_warp = ne > 0 && warp == 0;
+        const int w_first = ne > 0 ? 1 : 0;
+        const int i_begin = elite_warp ? 0 : ne + 2 * (warp - w_first);
+        const int i_step = elite_warp ? 2 : 2 * (nwarps - w_first);
+        const int i_end = elite_warp ? ne : nc;
+        const int hf = lane >> 4, hl = lane & 15;
+        const unsigned hmask = 0xffffu << (lane & 16);
+        for (int i0 = i_begin; i0 < i_end; i0 += i_step) {
+          const bool act = i0 + hf < i_end;  // (an idle half repeats the other's child)
+          const int i = act ? i0 + hf : i0;
+          const int slot = c0 + i;
+          const int n = base_n + slot;
+          const uint32_t* dr = DR + (size_t)i * nblk * 8;
+          uint32_t* child = reinterpret_cast<uint32_t*>(popn + slot * MS);
+          // Candidates: all members, or the island's.  Slot n of island c at
+          // position i is the island's rank-i member for i < min(E, m_c), found
+          // by this slot's lanes while the others build their children (a search
+          // of all islands before the children took 1.8 us of a 256-member
+          // generation's 7.3), else a child of two tournaments in the island.
+          const int* mem = nullptr;
+          int m = N, irank = -1;
+          bool elite = !isl && n < E;
+          if (isl) {
+            const int c = ilab[n], at = ipos[n];
+            mem = ilist + ioff[c];
+            m = ioff[c + 1] - ioff[c];
+            elite = at < min(E, m);
+            irank = at;
+          }
+          int pa_, pb_;
+          int split = LK;
+          if (elite) {
+            pa_ = pb_ = isl ? half_rank_list<FT>(fit, mem, m, irank, hmask, hl) : elites[n];
+          } else {
+            if (T_ <= 8) {  // eight lanes a tournament, a candidate each
+              const int t = lane & 7;
+              int c = -1;
+              FT v = (FT)0;
+              if (t < T_) {
+                c = (int)below(dr[((lane >> 3) & 1) * T_ + t], (uint32_t)m);
+                if (isl) c = mem[c];
+                v = fit[c];
+              }
+              for (int off = T_ > 4 ? 4 : 2; off > 0; off >>= 1) {
+                const int o = __shfl_xor_sync(hmask, c, off);
+                const FT ov = __shfl_xor_sync(hmask, v, off);
+                if (o >= 0 && (c < 0 || better_v(ov, o, v, c))) {
+                  c = o;
+                  v = ov;
+                }
+              }
+              pa_ = __shfl_sync(hmask, c, lane & 16);
+              pb_ = __shfl_sync(hmask, c, (lane & 16) + 8);
+            } else if (isl) {
+              pa_ = tournament_list(fit, mem, m, T_, dr);
+              pb_ = tournament_list(fit, mem, m, T_, dr + T_);
+            } else {
+              pa_ = tournament_lane(fit, N, T_, dr);
+              pb_ = tournament_lane(fit, N, T_, dr + T_);
+            }
+            if ((uint64_t)dr[2 * T_] < a.pc_thresh)
+              split = (1 + (int)below(dr[2 * T_ + 1], (uint32_t)(L - 1))) * K;
+          }
+          __syncwarp();
+          // parents' records from their owners, 16 bytes per lane and load
+          const int oa = nt_shift >= 0 ? pa_ >> nt_shift : pa_ / NT;
+          const int ob = nt_shift >= 0 ? pb_ >> nt_shift : pb_ / NT;
+          const uint32_t ra = dsmem_addr(POPp(cur) + (pa_ - oa * NT) * MS, oa);
+          const uint32_t rb = dsmem_addr(POPp(cur) + (pb_ - ob * NT) * MS, ob);
+  #pragma unroll 2
+          for (int v = hl; v < (MS >> 4); v += 16) {
+            const uint4 qa = ld_dsmem_v4(ra + 16 * v), qb = ld_dsmem_v4(rb + 16 * v);
+            // bytes below sp from A: the cut in X, and the same cut in INV
+            // (16-byte units never straddle XO); only one unit mixes the two
+            const int lo = 16 * v, sp = lo >= XO ? XO + split : split;
+            uint4 o;
+            if (lo + 16 <= sp) {
+              o = qa;
+            } else if (lo >= sp) {
+              o = qb;
+            } else {
+              o.x = merge_word(qa.x, qb.x, sp - lo);
+              o.y = merge_word(qa.y, qb.y, sp - lo - 4);
+              o.z = merge_word(qa.z, qb.z, sp - lo - 8);
+              o.w = merge_word(qa.w, qb.w, sp - lo - 12);
+            }
+            if (act) reinterpret_cast<uint4*>(child)[v] = o;
+          }
+          __syncwarp();
+          if (!elite && act) {
+            uint8_t* cx = reinterpret_cast<uint8_t*>(child);
+            for (int l = hl; l < L; l += 16) {
+              const int base = 2 * T_ + 2 + 3 * l;
+              if ((uint64_t)dr[base] < a.pm_thresh && K >= 2) {
+                const int i1 = (int)below(dr[base + 1], (uint32_t)K);
+                const int jj = (int)below(dr[base + 2], (uint32_t)(K - 1));
+                const int i2 = jj + (jj >= i1 ? 1 : 0);
+                uint8_t* xr = cx + l * K;
+                uint8_t* ir = cx + XO + l * K;
+                const uint8_t p1 = xr[i1], p2 = xr[i2];
+                xr[i1] = p2;
+                xr[i2] = p1;
+                if (p1 < K) ir[p1] = (uint8_t)i2;
+                if (p2 < K) ir[p2] = (uint8_t)i1;
+              }
+            }
+          }
+          __syncwarp();
+        }
       }
       __syncthreads();
     }
@@ -807,7 +978,6 @@ SolveShape solve_shape(const pa_ctx* ctx, int C, int maxnp, int threads) {
   s.nblk = (2 * c.tour + 2 + 3 * c.L + 7) / 8;
   s.C = C;
   s.NT = (c.N + C - 1) / C;
-  s.CH = std::max(1, std::min(s.NT, 16384 / (s.nblk * 32)));
   // record = X | INV, 16-byte aligned halves (records are copied 16 bytes
   // per lane); an odd number of 16-byte units per record spreads the
   // per-member inverse reads of one warp over the banks
@@ -844,12 +1014,19 @@ SolveShape solve_shape(const pa_ctx* ctx, int C, int maxnp, int threads) {
   b = (b + 15) & ~size_t(15);
   b += 2 * (size_t)s.NT * s.MS;
   b = (b + 15) & ~size_t(15);
-  b += (size_t)s.CH * s.nblk * 32;
   if (c.E > kSmallE) b += (f64 ? 8 : 4) * 32 * 64 + 4 * 32 * 64;  // elite candidates
   if (c.islands >= 2) {  // labels, positions, lists, offsets, sizes
     const size_t N4 = (size_t)((c.N + 3) & ~3);
     b += 4 * (3 * N4 + (size_t)((c.islands + 4) & ~3) + (size_t)c.islands);
   }
+  // draws: 16 KB, or (a CTA that has its SM to itself, no arrays behind these)
+  // all children's if there is room, so that they need no phase of their own
+  const size_t budget = (size_t)kSmemBudget - 64 * 4 - 16 - 64;
+  size_t room = 16384;
+  if (threads == kSolveThreads && c.islands < 2 && b + room < budget)
+    room = std::min<size_t>(budget - b, 65536);
+  s.CH = std::max(1, std::min(s.NT, (int)(room / (s.nblk * 32))));
+  b += (size_t)s.CH * s.nblk * 32;
   s.smem = (b + 15) & ~size_t(15);
   return s;
 }
