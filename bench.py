@@ -439,7 +439,7 @@ def run_ours(args):
                 "frac_of_cluster_sms": ks_gword / (peak_gword * ctas / n_sms) if ctas > 0
                 else None,
                 "note": "one instance: 201 dependent generations on one cluster, latency-bound"}
-    roofline_eval = {"bound": "alu", "kernel": "k_eval_f32_pilot (population fitness, FP32)",
+    roofline_eval = {"bound": "alu", "kernel": "k_eval_f32_lanes (population fitness, FP32)",
                      "achieved": achieved_gword, "peak": peak_gword, "unit": "Gword/s",
                      "frac": achieved_gword / peak_gword, "traffic": TRAFFIC_EVAL, "path": path,
                      "units_per_launch": nb, "words_per_unit": words,

@@ -21,10 +21,13 @@
 // bank-conflict free: lanes that read the same (l, u) row read the same
 // address (broadcast) and distinct u land in distinct banks (float2 loads,
 // RS/2 odd, K <= 16; scalar loads, RS odd, K <= 32).
-//   k_eval_f32_pilot (K <= 16, L <= 24): one thread per (chromosome, pilot)
-//     over all columns; chromosome tiles staged by bulk copies.
-//   k_eval_f32 (other shapes): the columns split in two shares taken by the
-//     two half-warps, chromosomes decoded from global memory.
+//   k_eval_f32_lanes (pa_eval_lanes.cuh): large calls, a lane per chromosome.
+//   k_eval_f32_pilot (smaller calls, K <= 16, L <= 24): one thread per
+//     (chromosome, pilot) over all columns; chromosome tiles staged by bulk
+//     copies.
+//   k_eval_f32 (smaller calls of other shapes): the columns split in two
+//     shares taken by the two half-warps, chromosomes decoded from global
+//     memory.
 //
 // FP64 kernel (parity path).  One thread per user (j, k) of a chromosome,
 // the oracle's operation order exactly: ascending-l sums, separately rounded

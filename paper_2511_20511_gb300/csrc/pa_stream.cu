@@ -1,6 +1,8 @@
 // pa_stream.cu -- population fitness (Sec. 3.2, Eq. 3-6) for instances whose
 // FP32 gain table does not fit in shared memory (e.g. 61 cells x 32 users:
-// 476 KB).
+// 476 KB): the kernel of small calls and the dispatch.  Large calls go to
+// k_eval_f32_chunk (K > 16) or k_eval_f32_lanes (K <= 16), which read the same
+// tiles.
 //
 // The BS-minor table is split into tiles of JT BS columns; tile t holds, for
 // every user (l, u), its gains at BSs t*JT .. t*JT+JT-1 (own-cell entries
