@@ -55,7 +55,7 @@ __device__ __forceinline__ ChunkPiece chunk_load(const uint8_t* x, int K, int l,
   ChunkPiece p;
   const uint8_t* r = x + l * K + k0;
   if (width == 16) {  // (K is a multiple of 16)
-    const uint4 q = __ldg(reinterpret_cast<const uint4*>(r));
+    const uint4 q = *reinterpret_cast<const uint4*>(r);
     p.v[0] = q.x;
     p.v[1] = q.y;
     p.v[2] = q.z;
@@ -63,14 +63,14 @@ __device__ __forceinline__ ChunkPiece chunk_load(const uint8_t* x, int K, int l,
   } else if (width == 4) {  // (K is a multiple of 4)
 #pragma unroll
     for (int w = 0; w < 4; ++w)
-      p.v[w] = k0 + 4 * w < K ? __ldg(reinterpret_cast<const uint32_t*>(r) + w) : 0u;
+      p.v[w] = k0 + 4 * w < K ? reinterpret_cast<const uint32_t*>(r)[w] : 0u;
   } else {
 #pragma unroll
     for (int w = 0; w < 4; ++w) {
       p.v[w] = 0;
 #pragma unroll
       for (int b = 0; b < 4; ++b)
-        if (k0 + 4 * w + b < K) p.v[w] |= (uint32_t)__ldg(r + 4 * w + b) << (8 * b);
+        if (k0 + 4 * w + b < K) p.v[w] |= (uint32_t)r[4 * w + b] << (8 * b);
     }
   }
   return p;
@@ -94,9 +94,8 @@ __device__ __forceinline__ void chunk_put(const ChunkPiece& p, uint32_t dst, int
 // cells), out[(tile * chunks + chunk) * chunk_words(K)].  Bytes that no row
 // fills name user 0.  Bound by its reads (32 rows a chromosome apart per load)
 // and its byte stores; one pass instead of one per column tile.
-__global__ void __launch_bounds__(kDecodeThreads) k_eval_decode(const uint8_t* __restrict__ pop,
-                                                                int64_t n, int L, int K, int width,
-                                                                uint32_t* __restrict__ out) {
+__global__ void __launch_bounds__(kDecodeThreads) k_eval_decode(const uint8_t* pop, int64_t n, int L,
+                                                                int K, int width, uint32_t* out) {
   extern __shared__ __align__(16) uint32_t inv[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = kDecodeThreads / 32;
   const int words = chunk_words(K), nch = chunk_count(L), kg = (K + 15) >> 4;
@@ -107,6 +106,8 @@ __global__ void __launch_bounds__(kDecodeThreads) k_eval_decode(const uint8_t* _
   const uint8_t* x = pop + min(tile * kLanesTile + lane, n - 1) * (L * K);
   constexpr int kU = 2;  // pieces on their way at once
   __syncthreads();
+  dependents_wait();
+  dependents_launch();
   for (int pc0 = warp; pc0 < kChunkCells * kg; pc0 += kU * nwarps) {
     ChunkPiece p[kU];
 #pragma unroll
@@ -133,8 +134,8 @@ __global__ void __launch_bounds__(kDecodeThreads) k_eval_decode(const uint8_t* _
 // adds its column tiles' partials in tile order into fit.
 template <int JT, int PPW, bool FIN>
 __global__ void __launch_bounds__(kChunkThreads, 1)
-    k_eval_f32_chunk(const LanesArgs a, const uint32_t* __restrict__ invg, float* __restrict__ fit,
-                     int* __restrict__ tickets) {
+    k_eval_f32_chunk(const LanesArgs a, const uint32_t* invg, float* fit,
+                     int* tickets) {
   extern __shared__ __align__(128) unsigned char smem[];
   // [0] the table's bulk copies; from 1: a buffer's chunk has landed; from
   // 1 + kChunkBufs: all warps have gathered it
@@ -182,11 +183,18 @@ __global__ void __launch_bounds__(kChunkThreads, 1)
     constexpr uint32_t kPart = 32768;
     for (uint32_t off = 0; off < bytes; off += kPart)
       bulk_g2s(smem_u32(T) + off, src + off, min(kPart, bytes - off), mb0);
-    for (int q = 0; q < kChunkBufs - 1 && q < chunks; ++q) issue(q);
   }
   for (int i = tid; i < LK; i += nthr) OWN[i] = __ldg(a.own + i);
   for (int i = tid; i < ((L + 15) & ~15); i += nthr) BN[i] = FIN && i < L ? __ldg(a.bn + i) : 0.f;
   __syncthreads();
+  // the table, which no kernel before this one in the call writes, is on its way
+  // while the inverses are still decoded
+  dependents_wait();
+  dependents_launch();
+  if (tid == 0) {
+    asm volatile("fence.proxy.async;" ::: "memory");  // inverses: stores, then bulk copies
+    for (int q = 0; q < kChunkBufs - 1 && q < chunks; ++q) issue(q);
+  }
 
   // A copy that has not landed after about a second sets the error flag; the
   // warp then waits for no more of them and the block runs to the end with
@@ -227,7 +235,7 @@ __global__ void __launch_bounds__(kChunkThreads, 1)
     if (n < a.n) {
       float s = mo ? __int_as_float(0x7f800000) : 0.f;
       for (int k = 0; k < a.ntile; ++k) {
-        const float x = __ldcg(a.fit + n * a.ntile + k);
+        const float x = *reinterpret_cast<const volatile float*>(a.fit + n * a.ntile + k);
         s = mo ? fminf(s, x) : s + x;
       }
       fit[n] = s;
@@ -358,12 +366,10 @@ cudaError_t run_chunk(const LanesArgs& a, const F32Tables& t, float* fit, int* t
   const int64_t want = std::max<int64_t>(1, (int64_t)per_sm * num_sms / a.ntile);
   const unsigned grid = (unsigned)(std::min(tiles, want) * a.ntile);
   (void)cudaGetLastError();  // drop a stale error of an earlier call
-  if (fin)
-    k_eval_f32_chunk<JT, PPW, true><<<grid, threads, smem, st>>>(a, t.inv, fit, tickets);
-  else
-    k_eval_f32_chunk<JT, PPW, false><<<grid, threads, smem, st>>>(a, t.inv, fit, tickets);
+  e = launch_early(fin ? k_eval_f32_chunk<JT, PPW, true> : k_eval_f32_chunk<JT, PPW, false>, grid,
+                   (unsigned)threads, smem, st, a, t.inv, fit, tickets);
   count_launch();
-  return cudaGetLastError();
+  return e;
 }
 
 }  // namespace
@@ -374,7 +380,7 @@ cudaError_t run_chunk(const LanesArgs& a, const F32Tables& t, float* fit, int* t
 // device memory for the inverses of kChunkSlab chromosomes: the context keeps
 // them, at most 256 MB or so).  *summed: fit is written, else the caller adds
 // the partials.  Where a block has few tiles, tickets save the launch that adds
-// the partials (4 us of a generation's 78 at n = 2048); with many, the fence
+// the partials (4 us of a generation's 78 at n = 2048, all launches ordinary); with many, the fence
 // behind each tile costs more (2^17: 2,428 us against 2,348).
 cudaError_t launch_eval_chunk(pa_ctx* ctx, const uint8_t* pop, int64_t n, float* fit,
                               bool* summed, cudaStream_t st) {
@@ -442,10 +448,9 @@ cudaError_t launch_eval_chunk(pa_ctx* ctx, const uint8_t* pop, int64_t n, float*
     const int width = K % 16 == 0 && base % 16 == 0 ? 16 : K % 4 == 0 && base % 4 == 0 ? 4 : 1;
     const int64_t tiles = (a.n + kLanesTile - 1) / kLanesTile;
     (void)cudaGetLastError();  // drop a stale error of an earlier call
-    k_eval_decode<<<(unsigned)(tiles * nch), kDecodeThreads, 4 * (size_t)a.inv_words, st>>>(
-        x, a.n, L, K, width, t.inv);
+    cudaError_t e = launch_early(k_eval_decode, (unsigned)(tiles * nch), kDecodeThreads,
+                                 4 * (size_t)a.inv_words, st, x, a.n, L, K, width, t.inv);
     count_launch();
-    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     switch (t.JT * 10 + PPW) {
       case 161: e = run_chunk<16, 1>(a, t, fit + n0, tickets, fin, b, ctx->num_sms, st); break;

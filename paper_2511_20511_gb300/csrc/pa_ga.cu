@@ -143,7 +143,7 @@ __device__ void ga_elites(const GaArgs& a, int* elites, int* wi, FT* wv) {
 #pragma unroll
   for (int r = 0; r < kGaCache; ++r) {
     const int i = tid + kGaThreads * r;
-    vc[r] = i < a.N ? __ldg(fit + i) : (FT)0;
+    vc[r] = i < a.N ? fit[i] : (FT)0;
   }
   for (int e = 0; e < a.E; ++e) {
     int best = -1;
@@ -160,7 +160,7 @@ __device__ void ga_elites(const GaArgs& a, int* elites, int* wi, FT* wv) {
       bool skip = false;
       for (int f = 0; f < e; ++f) skip |= elites[f] == i;
       if (skip) continue;
-      const FT v = __ldg(fit + i);
+      const FT v = fit[i];
       if (better_val(v, i, bv, best)) {
         best = i;
         bv = v;
@@ -190,26 +190,34 @@ __device__ void ga_elites(const GaArgs& a, int* elites, int* wi, FT* wv) {
   __syncthreads();
   const int64_t LK = (int64_t)a.L * a.K;
   for (int e = warp; e < a.E; e += kGaWarps) {
-    const uint8_t* __restrict__ src = a.pop + (int64_t)elites[e] * LK;
-    uint8_t* __restrict__ dst = a.next + (int64_t)e * LK;
-    for (int64_t i = lane; i < LK; i += 32) dst[i] = src[i];
+    const uint8_t* src = a.pop + (int64_t)elites[e] * LK;
+    uint8_t* dst = a.next + (int64_t)e * LK;
+    constexpr int kU = 8;  // loads on their way at once
+    for (int64_t i0 = lane; i0 < LK; i0 += 32 * kU) {
+      uint8_t x[kU];
+#pragma unroll
+      for (int u = 0; u < kU; ++u)
+        if (i0 + 32 * u < LK) x[u] = src[i0 + 32 * u];
+#pragma unroll
+      for (int u = 0; u < kU; ++u)
+        if (i0 + 32 * u < LK) dst[i0 + 32 * u] = x[u];
+    }
   }
 }
 
 // Bytes i .. i+W-1 of a child: from A below split, from B from there on (the
 // unit holding the cut byte by byte).
 template <typename V>
-__device__ __forceinline__ void ga_copy(uint8_t* child, const uint8_t* __restrict__ A,
-                                        const uint8_t* __restrict__ B, int LK, int split,
-                                        int lane) {
+__device__ __forceinline__ void ga_copy(uint8_t* child, const uint8_t* A, const uint8_t* B, int LK,
+                                        int split, int lane) {
   constexpr int W = (int)sizeof(V);
 #pragma unroll 4
   for (int i = lane * W; i < LK; i += 32 * W) {
     if (i + W <= split || i >= split) {
       const uint8_t* src = i + W <= split ? A : B;
-      *reinterpret_cast<V*>(child + i) = __ldg(reinterpret_cast<const V*>(src + i));
+      *reinterpret_cast<V*>(child + i) = *reinterpret_cast<const V*>(src + i);
     } else {
-      for (int j = i; j < i + W; ++j) child[j] = __ldg((j < split ? A : B) + j);
+      for (int j = i; j < i + W; ++j) child[j] = (j < split ? A : B)[j];
     }
   }
 }
@@ -223,7 +231,9 @@ __device__ __forceinline__ void ga_copy(uint8_t* child, const uint8_t* __restric
 // load, a parent load and the stores (61 x 32, N = 2048, cold caches: 17 us; with
 // a block per eight children, the elites searched by the first of them before
 // its children, tournaments re-reading the fitness at each comparison and rows
-// copied bytewise: 25.4 us).
+// copied bytewise: 25.4 us).  Launched early: a block may start while the
+// evaluation's last blocks run, and has its first children's draws by the time
+// the fitness is there.
 template <typename FT>
 __global__ void __launch_bounds__(kGaThreads) k_ga_step(const GaArgs a, int width) {
   extern __shared__ __align__(16) unsigned char gsm[];
@@ -233,6 +243,8 @@ __global__ void __launch_bounds__(kGaThreads) k_ga_step(const GaArgs a, int widt
   const FT* fit = static_cast<const FT*>(a.fit);
   const int E = a.E, T = a.tour, LK = a.L * a.K;
   if (E > 0 && blockIdx.x == gridDim.x - 1) {
+    dependents_wait();
+    dependents_launch();
     ga_elites<FT>(a, elites, wi, wv);
     return;
   }
@@ -242,14 +254,19 @@ __global__ void __launch_bounds__(kGaThreads) k_ga_step(const GaArgs a, int widt
   unsigned char* mine = gsm + (size_t)warp * (nblk * 32 + ((LK + 15) & ~15));
   uint32_t* dr = reinterpret_cast<uint32_t*>(mine);
   uint8_t* child = mine + nblk * 32;
-  for (int n = E + blockIdx.x * kGaWarps + warp; n < a.N; n += nw) {
+  const int first = E + blockIdx.x * kGaWarps + warp;
+  for (int n = first; n < a.N; n += nw) {
     gen_child_draws_from(dr, n, 1, nblk, a.seed, (uint64_t)a.gen, 0, lane, 32);
     __syncwarp();
+    if (n == first) {  // the first draws need nothing of the evaluation
+      dependents_wait();
+      dependents_launch();
+    }
     int par[2];
     if (T <= 16) {  // one tournament per half-warp
       const int h = lane >> 4, t = lane & 15;
       int c = t < T ? (int)below(dr[h * T + t], (uint32_t)a.N) : -1;
-      FT v = c >= 0 ? __ldg(fit + c) : (FT)0;
+      FT v = c >= 0 ? fit[c] : (FT)0;
       lanes_best(c, v, 16);
       par[0] = __shfl_sync(0xffffffffu, c, 0);
       par[1] = __shfl_sync(0xffffffffu, c, 16);
@@ -260,7 +277,7 @@ __global__ void __launch_bounds__(kGaThreads) k_ga_step(const GaArgs a, int widt
         FT bv = (FT)0;
         for (int t = lane; t < T; t += 32) {
           const int c = (int)below(dr[h * T + t], (uint32_t)a.N);
-          const FT v = __ldg(fit + c);
+          const FT v = fit[c];
           if (better_val(v, c, bv, best)) {
             best = c;
             bv = v;
@@ -672,12 +689,10 @@ cudaError_t launch_ga_step(const pa_ctx* ctx, const uint8_t* pop, const void* fi
     capped[f64].fetch_or(bit);
   }
   (void)cudaGetLastError();  // drop a stale error of an earlier call
-  if (f64)
-    k_ga_step<double><<<blocks, kGaThreads, smem, st>>>(a, width);
-  else
-    k_ga_step<float><<<blocks, kGaThreads, smem, st>>>(a, width);
+  const cudaError_t e = launch_early(f64 ? k_ga_step<double> : k_ga_step<float>, (unsigned)blocks,
+                                     kGaThreads, smem, st, a, width);
   count_launch();
-  return cudaGetLastError();
+  return e;
 }
 
 size_t seed_smem(int L, int K, int kk, int threads, int C) {
