@@ -174,6 +174,8 @@ __global__ void __launch_bounds__(kPilotThreads, 4) k_eval_f32_pilot(const Pilot
     mbar_init(mb0, 1);
     mbar_init(mb0 + 8, 1);
     s_timeout = 0;
+    issue(blockIdx.x, 0);  // (on their way while the table is staged)
+    issue(blockIdx.x + (int64_t)gridDim.x, 1);
   }
   {
     const float4* s4 = reinterpret_cast<const float4*>(a.tab);
@@ -186,8 +188,6 @@ __global__ void __launch_bounds__(kPilotThreads, 4) k_eval_f32_pilot(const Pilot
     for (int i = tid; i < NTK * NJ / 4; i += blockDim.x) reinterpret_cast<uint32_t*>(INVT)[i] = 0;
   }
   __syncthreads();
-  issue(blockIdx.x, 0);
-  issue(blockIdx.x + (int64_t)gridDim.x, 1);
 
   const int c_me = tid / K;
   const int KRS = K * a.RS;
@@ -445,7 +445,7 @@ cudaError_t run_f32(const F32Args& a, const F32Launch& s, int num_sms, cudaStrea
 // Block shape of k_eval_f32_pilot: NT members (NT*L*K a multiple of 16 so
 // that a full tile is one bulk copy), one thread per (member, pilot).
 struct PilotLaunch {
-  int NT, xbytes;
+  int NT, unit, xbytes;
   size_t smem;
 };
 PilotLaunch pilot_shape(int L, int K, int RS, int NJ) {
@@ -454,6 +454,7 @@ PilotLaunch pilot_shape(int L, int K, int RS, int NJ) {
   int g = 16;
   while (LK % g) g >>= 1;
   const int m = 16 / g;
+  s.unit = m;
   s.NT = std::max(m, (kPilotThreads / K) / m * m);
   s.xbytes = (s.NT * LK + 20 + 15) & ~15;  // +20: a row reads up to 5 words from its first
   const size_t tab = (((size_t)LK * RS + 3) / 4) * 4;
@@ -461,6 +462,20 @@ PilotLaunch pilot_shape(int L, int K, int RS, int NJ) {
   s.smem = 4 * (tab + ((LK + 3) & ~size_t(3)) + ((L + 3) & ~3) + ((NTK * (NJ / 2) + 3) & ~size_t(3))) +
            ((NTK * NJ + 15) & ~size_t(15)) + 2 * (size_t)s.xbytes;
   return s;
+}
+
+// Members per tile of a call: the block's NT, or for fewer members than all SMs'
+// blocks take, what spreads them over the SMs (a multiple of unit); the block
+// keeps its threads and shared memory.  A block of few members has its chain of
+// decode, gathers and sums shorter by the data path's share.
+// Per call, back to back, full blocks / spread (and the pilot kernel's chromosome
+// copies issued before the table's staging instead of behind it):
+//   19 x 10  n = 256: 10.2 / 8.2 us   2048: 10.3 / 8.2
+//   37 x 13  n = 256: 12.3 / 8.2 us   1024: 12.3 / 10.4
+//   19 x 24  n = 256: 10.3 / 8.2 us   16 x 16  n = 32: 8.2 / 6.2
+int spread_members(int64_t n, int NT, int unit, int num_sms) {
+  const int64_t per = (n + num_sms - 1) / num_sms;
+  return (int)std::min<int64_t>(NT, std::max<int64_t>(1, (per + unit - 1) / unit) * unit);
 }
 
 bool pilot_kernel_applies(int NJ, int vec, int K) { return vec == 2 && NJ <= 24 && K <= 16; }
@@ -552,7 +567,7 @@ cudaError_t launch_eval_f32(pa_ctx* ctx, const uint8_t* pop, int64_t n, float* f
     a.L = L;
     a.K = K;
     a.RS = t.RS;
-    a.NT = s.NT;
+    a.NT = spread_members(n, s.NT, s.unit, ctx->num_sms);
     a.tab_floats = (((int64_t)L * K * t.RS + 3) / 4) * 4;
     a.xbytes = s.xbytes;
     a.stall = ctx->test_stall;
@@ -574,8 +589,8 @@ cudaError_t launch_eval_f32(pa_ctx* ctx, const uint8_t* pop, int64_t n, float* f
   a.L = L;
   a.K = K;
   a.RS = t.RS;
-  a.NT = s.NT;
-  a.NTK = s.NT * K;
+  a.NT = spread_members(n, s.NT, 1, ctx->num_sms);
+  a.NTK = a.NT * K;
   a.tab_floats = (((int64_t)L * K * t.RS + 3) / 4) * 4;
   a.M = t.M;
   a.pc = t.pc;
