@@ -10,8 +10,6 @@ namespace pa {
 // Small calls stay with the kernels of fewer chromosomes per block
 // (pa_fitness.cu, pa_stream.cu), which spread them over more SMs and start
 // sooner.  Measured on GB300, those kernels against these:
-//   19 x 10  n = 1024: 10.3 / 12.4 us   4096: 12.4 / 12.4   65536: 51.8 / 43.3
-//   7 x 16   n = 8192: 8.3 / 9.0 us    16384: 11.3 / 10.3   65536: 26.8 / 19.6
 //   37 x 13  n = 1024: 12.4 / 20.6 us   4096: 25.8 / 20.7   65536: 240 / 162
 //   61 x 16 (column tiles)  n = 1024: 22.7 / 24.7 us   4096: 62.0 / 55.7
 //   61 x 32 (column tiles, chunks)  n = 2^17: 2,853 / 2,348 us
@@ -23,6 +21,20 @@ bool lanes_applies(const pa_ctx* ctx, int64_t n) {
   const int64_t tiles = (n + kLanesTile - 1) / kLanesTile;
   if (n * LK * L < kLanesMinWords) return false;
   return t.streamed ? tiles * t.ntile >= ctx->num_sms : 5 * tiles >= 4 * ctx->num_sms;
+}
+
+// Tiles per SM from which it pays against the thread-per-(chromosome, pilot)
+// kernel (K <= 16, L <= 24), x 10.  That kernel does no work for pad columns
+// where L is a multiple of 4, and many pilots make this one's blocks few per SM.
+// Measured, that kernel / this one:
+//   19 x 10  n = 4096: 12.3 / 12.3 us   19,456: 22.0 / 18.6   48,000: 39.3 / 35.1
+//   10 x 16  n = 13,000: 11.5 / 12.5    19,456: 14.6 / 12.5
+//   16 x 16  n = 4096: 10.3 / 12.4      19,456: 20.8 / 24.8   80,000: 70.0 / 68.7
+//   20 x 13  n = 4096: 10.3 / 13.8      19,456: 22.7 / 24.8   48,000: 47.3 / 43.3
+//   24 x 4   n = 6144: 12.3 / 10.3      (K <= 8: never slower)
+// With one block per SM (24 x 16) it stays behind: n = 300,000: 427 / 469 us.
+static int64_t lanes_line(int L, int K) {
+  return K <= 8 ? 8 : K > 12 && L % 4 == 0 ? 100 : 40;
 }
 
 // cudaErrorNotSupported where the kernel does not apply: a small call, or its
@@ -74,6 +86,9 @@ cudaError_t launch_eval_lanes(pa_ctx* ctx, const uint8_t* pop, int64_t n, float*
   // since all warps of an SM get an equal part of its issue slots; evaluation
   // warps: the units (pilot, share) in equal rounds
   const int fit_blocks = std::max(1, (int)((size_t)kSmemBudget / (b + 1024)));
+  if (!t.streamed && K <= 16 && L <= 24 &&
+      (fit_blocks < 2 || 10 * tiles < lanes_line(L, K) * ctx->num_sms))
+    return cudaErrorNotSupported;
   const int maxw = std::min(32, 36 / std::min(fit_blocks, 6));
   const int units = K * JS;
   const int unitw = L * (2 + 3 * W) + 22 * W, helpw = 4 * LK + 4 * K * a.NPR + 200;

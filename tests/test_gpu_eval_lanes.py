@@ -60,7 +60,7 @@ def _chunks(B, ctx, pop, step):
 @pytest.mark.parametrize("mode,obj", [(1, 0), (0, 0), (1, 1)])
 def test_large_call_equals_small_calls(B, oracle, L, K, mode, obj):
     beta = _instance(L, K)
-    n = max(WORDS // (L * L * K) + 1, 6001) | 1  # odd: a ragged last tile
+    n = max(WORDS // (L * L * K) + 1, 50001) | 1  # odd: a ragged last tile
     cfg = _cfg(B, L, K, mode, obj)
     ctx = B.pa_create(cfg, beta)
     try:
