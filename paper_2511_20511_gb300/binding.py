@@ -131,6 +131,36 @@ def _check(st, ctx=None):
         raise PaError(st, msg)
 
 
+class _Handle(C.c_void_p):
+    """Opaque pointer of the library.  With `destroy` set (the name of the
+    function that frees it) it is freed when its last reference goes; `keep`
+    is what has to outlive it.  Device addresses handed out (DevicePtr) hold
+    such a reference, so memory read through them outlives the Python object
+    it was asked from."""
+
+    destroy = None
+    keep = None
+
+    def __del__(self):
+        try:
+            if self.destroy and self.value:
+                getattr(lib(), self.destroy)(self)
+        except Exception:
+            pass
+
+
+class DevicePtr(int):
+    """Device address inside an object of the library (`owner`, its handle):
+    an int that keeps that object, and so the memory, alive -- in a
+    __cuda_array_interface__, for instance.  An explicit close() or
+    pa_destroy frees the memory all the same."""
+
+    def __new__(cls, value, owner):
+        p = super().__new__(cls, value)
+        p.owner = owner
+        return p
+
+
 def _host_ptr(a):
     return None if a is None else a.ctypes.data_as(C.c_void_p)
 
@@ -172,7 +202,7 @@ def pa_create(cfg, beta, user_xy_mm=None, bs_xy_mm=None, stream=None):
         raise ValueError("user_xy_mm must be (L, K, 2)")
     if b is not None and b.shape != (cfg.L, 2):
         raise ValueError("bs_xy_mm must be (L, 2)")
-    out = C.c_void_p()
+    out = _Handle()
     st = lib().pa_create(C.byref(cfg), _host_ptr(beta), _host_ptr(u), _host_ptr(b),
                          _stream_handle(stream), C.byref(out))
     _check(st, None)
@@ -216,6 +246,8 @@ def pa_solve_cluster_ctas(ctx):
 
 
 def pa_destroy(ctx):
+    if isinstance(ctx, _Handle):
+        ctx.destroy = None
     lib().pa_destroy(ctx)
 
 
@@ -270,10 +302,11 @@ def pa_set_population(ctx, pop, generation):
 
 
 def pa_population_device(ctx):
+    """Addresses of the resident population and its fitness; they hold ctx."""
     p = C.c_void_p()
     f = C.c_void_p()
     _check(lib().pa_population_device(ctx, C.byref(p), C.byref(f)), ctx)
-    return p.value, f.value
+    return tuple(None if v.value is None else DevicePtr(v.value, ctx) for v in (p, f))
 
 
 def pa_validate_population(ctx, pop, n=None):
@@ -305,13 +338,16 @@ def pa_get_islands(ctx, n):
 
 # ------------------------------------------------------------------ convenience
 class Context:
-    """Owns one pa_ctx.  Methods mirror the C entry points."""
+    """Owns one pa_ctx, destroyed by close(), or once neither this object nor
+    an address of the context's memory is referenced any more.  Methods mirror
+    the C entry points."""
 
     def __init__(self, cfg, beta, user_xy_mm=None, bs_xy_mm=None, stream=None):
         self.cfg = cfg
         self.L, self.K, self.N = cfg.L, cfg.K, cfg.N
         self.fit_dtype = np.float64 if cfg.prec == PA_FP64 else np.float32
         self.handle = pa_create(cfg, beta, user_xy_mm, bs_xy_mm, stream)
+        self.handle.destroy = "pa_destroy"
 
     def close(self):
         if self.handle:
@@ -323,12 +359,6 @@ class Context:
 
     def __exit__(self, *exc):
         self.close()
-
-    def __del__(self):
-        try:
-            self.close()
-        except Exception:
-            pass
 
     def torch_fit_dtype(self):
         import torch
@@ -412,12 +442,13 @@ class Batch:
                 self._keep += [u, s]
                 ux[i] = u.ctypes.data
                 bx[i] = s.ctypes.data
-        out = C.c_void_p()
+        out = _Handle()
         st = lib().pa_batch_create(n, C.cast(self.cfgs, C.c_void_p), C.cast(betas, C.c_void_p),
                                    C.cast(ux, C.c_void_p) if have_pos else None,
                                    C.cast(bx, C.c_void_p) if have_pos else None,
                                    _stream_handle(stream), C.byref(out))
         _check(st, None)
+        out.destroy = "pa_batch_destroy"
         self.handle = out
         self.offsets = np.cumsum([0] + [L * K for L, K in self.shapes])
 
@@ -483,20 +514,16 @@ class Batch:
         self._keep.append((b, u, s))
 
     def context(self, i):
-        out = C.c_void_p()
+        out = _Handle()
         self._bcheck(lib().pa_batch_context(self.handle, int(i), C.byref(out)))
+        out.keep = self.handle
         return out
 
     def close(self):
         if self.handle:
+            self.handle.destroy = None
             lib().pa_batch_destroy(self.handle)
             self.handle = None
-
-    def __del__(self):
-        try:
-            self.close()
-        except Exception:
-            pass
 
 
 class Server:
