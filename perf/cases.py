@@ -175,11 +175,9 @@ def prepare(case, seed):
 
 
 class _DeviceBytes:
-    """The context's resident population, seen by torch without a copy; the
-    view keeps the context, and so the memory, alive."""
+    """The context's resident population, seen by torch without a copy."""
 
-    def __init__(self, ctx, ptr, shape):
-        self.ctx = ctx
+    def __init__(self, ptr, shape):
         self.__cuda_array_interface__ = {"shape": shape, "typestr": "|u1", "data": (ptr, False),
                                          "version": 2}
 
@@ -193,7 +191,7 @@ def run(state):
         best, fitness = ctx.solve(state["G"])
         ptr, _ = B.pa_population_device(ctx.handle)
         if ptr not in state["views"]:
-            state["views"][ptr] = torch.as_tensor(_DeviceBytes(ctx, ptr, (ctx.N, ctx.L, ctx.K)),
+            state["views"][ptr] = torch.as_tensor(_DeviceBytes(ptr, (ctx.N, ctx.L, ctx.K)),
                                                   device=DEV)
         return {"best": best, "fitness": fitness, "population": state["views"][ptr]}
     if kind == "batch":
