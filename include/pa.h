@@ -111,8 +111,9 @@ typedef struct {
 /*
  * Testing the bounded waits.  With this flag the context's next FP32
  * evaluation that stages chromosome tiles by bulk copies announces the
- * copies to its mbarriers but never issues them: every block's wait gives
- * up after about a second (the kernel returns normally, nothing faults),
+ * copies to its mbarriers but never issues them: each wait for one gives
+ * up after about a second (the kernel returns normally after a few such
+ * waits, nothing faults),
  * and the next synchronous call reports PA_ETIMEOUT.  One-shot: later
  * evaluations of the context run normally.  The paper has no counterpart.
  */

@@ -449,13 +449,17 @@ __global__ void __maxnreg__(kLanesRegs) k_eval_f32_lanes(const LanesArgs a) {
     mbar_wait(mb0 + 8 * m, ph);  // a bounded chance to land before its buffer is left
     late = true;
   };
-  // the block's own warps always arrive, a late one after two of its waits:
-  // the bound here is a net, several times that
+  // The block's own warps always arrive, a late one after two of its waits:
+  // the bound here is a net, several times that.  A late warp waits for the
+  // others as before: one that ran ahead would complete phases that they have
+  // not seen, and they would sit their whole bound out (a call whose copies
+  // never come returned after 9.7 s that way).
+  bool lost = false;
   auto wait_warps = [&](int m, int i) {
-    for (int k = 0; k < 8 && !late; ++k)
+    for (int k = 0; k < 8 && !lost; ++k)
       if (mbar_wait(mb0 + 8 * m, (uint32_t)i & 1)) return;
-    if (lane == 0 && !late && a.err_flag) atomicExch(a.err_flag, 1);
-    late = true;
+    if (lane == 0 && !lost && a.err_flag) atomicExch(a.err_flag, 1);
+    lost = true;
   };
   auto arrive = [&](int m) {
     __syncwarp();
