@@ -376,7 +376,7 @@ cudaError_t run_chunk(const LanesArgs& a, const F32Tables& t, float* fit, int* t
 
 // Column-tiled tables with K > 16 (scalar rows): the fitness of n chromosomes;
 // t.partial holds n * ntile values.  cudaErrorNotSupported for other tables,
-// small calls (lanes_applies), or where it does not fit (shared memory, or
+// small calls (tiles_pay), or where it does not fit (shared memory, or
 // device memory for the inverses of kChunkSlab chromosomes: the context keeps
 // them, at most 256 MB or so).  *summed: fit is written, else the caller adds
 // the partials.  Where a block has few tiles, tickets save the launch that adds
@@ -386,8 +386,8 @@ cudaError_t launch_eval_chunk(pa_ctx* ctx, const uint8_t* pop, int64_t n, float*
                               bool* summed, cudaStream_t st) {
   F32Tables& t = ctx->t32;
   const int L = ctx->cfg.L, K = ctx->cfg.K, LK = L * K;
-  if (!t.streamed || t.vec != 1 || !lanes_applies(ctx, n)) return cudaErrorNotSupported;
   const int PPW = K <= kChunkThreads / 32 ? 1 : 2;
+  if (!t.streamed || t.vec != 1 || !tiles_pay(ctx, n)) return cudaErrorNotSupported;
   if (t.JT == 16 && PPW != 1) return cudaErrorNotSupported;  // (too many sums per thread)
   LanesArgs a{};
   a.ntile = t.ntile;

@@ -7,43 +7,39 @@
 
 namespace pa {
 
-// Small calls stay with the kernels of fewer chromosomes per block
-// (pa_fitness.cu, pa_stream.cu), which spread them over more SMs and start
-// sooner.  Measured on GB300, those kernels against these:
-//   37 x 13  n = 1024: 12.4 / 20.6 us   4096: 25.8 / 20.7   65536: 240 / 162
-//   61 x 16 (column tiles)  n = 1024: 22.7 / 24.7 us   4096: 62.0 / 55.7
-//   61 x 32 (column tiles, chunks)  n = 2^17: 2,853 / 2,348 us
-// so the line lies where most SMs get a tile of 32 and the call gathers 12
-// million table words.
-bool lanes_applies(const pa_ctx* ctx, int64_t n) {
-  const F32Tables& t = ctx->t32;
-  const int64_t L = ctx->cfg.L, LK = L * ctx->cfg.K;
-  const int64_t tiles = (n + kLanesTile - 1) / kLanesTile;
-  if (n * LK * L < kLanesMinWords) return false;
-  return t.streamed ? tiles * t.ntile >= ctx->num_sms : 5 * tiles >= 4 * ctx->num_sms;
-}
-
-// Tiles per SM from which it pays against the thread-per-(chromosome, pilot)
-// kernel (K <= 16, L <= 24), x 10.  That kernel does no work for pad columns
-// where L is a multiple of 4, and many pilots make this one's blocks few per SM.
-// Measured, that kernel / this one:
-//   19 x 10  n = 4096: 12.3 / 12.3 us   19,456: 22.0 / 18.6   48,000: 39.3 / 35.1
-//   10 x 16  n = 13,000: 11.5 / 12.5    19,456: 14.6 / 12.5
-//   16 x 16  n = 4096: 10.3 / 12.4      19,456: 20.8 / 24.8   80,000: 70.0 / 68.7
-//   20 x 13  n = 4096: 10.3 / 13.8      19,456: 22.7 / 24.8   48,000: 47.3 / 43.3
-//   24 x 4   n = 6144: 12.3 / 10.3      (K <= 8: never slower)
-// With one block per SM (24 x 16) it stays behind: n = 300,000: 427 / 469 us.
-static int64_t lanes_line(int L, int K) {
-  return K <= 8 ? 8 : K > 12 && L % 4 == 0 ? 100 : 40;
+// Time (us) of a resident-table call by this kernel, to be held against
+// small_eval_us (pa_fitness.cu).  Both kernels' times are staircases: what counts
+// is the whole tiles of the busiest SM (m) and how often its blocks come round
+// (`later` rounds beyond the first), so that a call changes sides several times
+// as it grows (43 x 6, small calls' kernel / this one: 1.2 tiles per SM 16.3 /
+// 21.9 us, 1.5: 23.0 / 21.8, 2.5: 27.8 / 31.7, 5: 50.5 / 49.2), and a line in the
+// count alone sends calls to the slower one.  The terms: launch and fixed chain,
+// buffers to fill, code to fetch (it grows with the columns), a unit's chain over
+// the cells, gathers and decoding per tile, later rounds' chains.  Fitted to
+// graph-replayed calls of 83 shapes (2 to 48 cells, 3 to 64 users) at 29 counts
+// each: the kernel chosen is 0.8 % above the faster one in the mean (lines in the
+// count: 2.5 %).  On 750 other calls of random shapes and counts: 0.4 %, and with
+// lines 15 had been slower by 8 % and more than before there was a second kernel,
+// up to 1.49 times.
+static double lanes_us(const LanesArgs& a, int cols, int rounds, size_t smem, int64_t tiles,
+                       int num_sms) {
+  const int threads = (a.EW + a.NH) * 32;
+  const int per_sm = std::max(1, std::min({(int)(kSmemPerSm / (smem + 1024 + 128)),
+                                           65536 / (kLanesRegs * threads), 2048 / threads}));
+  const double m = (double)((tiles + num_sms - 1) / num_sms), L = a.L, LK = L * a.K;
+  const double later = (double)(((int64_t)m - 1) / per_sm);
+  const double chain = 0.01 * rounds * L;
+  return 4.45 + 1.64e-5 * smem + 1.47e-3 * cols * cols + 2.35 * chain +
+         (2.74e-4 * L * LK + 5.8e-3 * LK) * m + 4.42 * later * chain;
 }
 
 // cudaErrorNotSupported where the kernel does not apply: a small call, or its
 // buffers exceed shared memory.  Resident tables write fit[n]; column-tiled
-// ones partial[n][ntile].
+// ones partial[n][ntile] (tiles_pay, pa_stream.cu).
 cudaError_t launch_eval_lanes(pa_ctx* ctx, const uint8_t* pop, int64_t n, float* out,
                               cudaStream_t st) {
-  if (!lanes_applies(ctx, n)) return cudaErrorNotSupported;
   const F32Tables& t = ctx->t32;
+  if (t.streamed && !tiles_pay(ctx, n)) return cudaErrorNotSupported;
   const int L = ctx->cfg.L, K = ctx->cfg.K, LK = L * K;
   const int64_t tiles = (n + kLanesTile - 1) / kLanesTile;
   LanesArgs a{};
@@ -86,9 +82,6 @@ cudaError_t launch_eval_lanes(pa_ctx* ctx, const uint8_t* pop, int64_t n, float*
   // since all warps of an SM get an equal part of its issue slots; evaluation
   // warps: the units (pilot, share) in equal rounds
   const int fit_blocks = std::max(1, (int)((size_t)kSmemBudget / (b + 1024)));
-  if (!t.streamed && K <= 16 && L <= 24 &&
-      (fit_blocks < 2 || 10 * tiles < lanes_line(L, K) * ctx->num_sms))
-    return cudaErrorNotSupported;
   const int maxw = std::min(32, 36 / std::min(fit_blocks, 6));
   const int units = K * JS;
   const int unitw = L * (2 + 3 * W) + 22 * W, helpw = 4 * LK + 4 * K * a.NPR + 200;
@@ -100,6 +93,15 @@ cudaError_t launch_eval_lanes(pa_ctx* ctx, const uint8_t* pop, int64_t n, float*
   }
   // warps left over decode
   while (a.EW + a.NH < maxw && a.NH < 6 && a.NH >= 3) ++a.NH;
+  a.L = L;
+  a.K = K;
+  if (!t.streamed) {
+    // scalar rows of few cells: below 12 million gathered words never faster
+    // (2 x 36, n = 8,728: 6.2 / 10.1 us; 7 x 20, n = 8,243: 7.7 / 8.8)
+    if (t.vec == 1 && n * LK * L < 12000000) return cudaErrorNotSupported;
+    const double us = lanes_us(a, cols, (units + a.EW - 1) / a.EW, b, tiles, ctx->num_sms);
+    if (1.02 * us >= small_eval_us(ctx, n)) return cudaErrorNotSupported;
+  }
   a.pop = pop;
   a.n = n;
   a.fit = out;
@@ -107,8 +109,6 @@ cudaError_t launch_eval_lanes(pa_ctx* ctx, const uint8_t* pop, int64_t n, float*
   a.own = t.own;
   a.bn = t.bn;
   a.err_flag = t.err_flag;
-  a.L = L;
-  a.K = K;
   a.M = t.M;
   a.pc = t.pc;
   a.obj = ctx->cfg.objective;

@@ -47,11 +47,9 @@
 
 namespace pa {
 
-constexpr int kLanesTile = 32;        // chromosomes per tile
 constexpr int kLanesRegs = 56;        // 36 warps per SM
 constexpr int kLanesMaxNP = 6;        // column pairs per unit at most
 constexpr int kLanesMaxNC = 48;       // columns per block at most
-constexpr int64_t kLanesMinWords = 12000000;  // table words a call gathers, at least
 
 struct LanesArgs {
   const uint8_t* pop;
@@ -80,13 +78,6 @@ struct LanesArgs {
 using LanesDispatch = cudaError_t(int NC, const LanesArgs& a, size_t smem, int num_sms,
                                   int64_t tiles, cudaStream_t st);
 LanesDispatch lanes_dispatch_fin2, lanes_dispatch_fin1, lanes_dispatch_asy2, lanes_dispatch_asy1;
-
-// Whether a call of n chromosomes is large enough for these kernels
-// (pa_eval_lanes.cu).
-bool lanes_applies(const pa_ctx* ctx, int64_t n);
-
-// Resident blocks per SM of a kernel at a launch shape, cached (pa_fitness.cu).
-int cached_occupancy(const void* fn, int threads, size_t smem, cudaError_t* err);
 
 namespace {
 
@@ -442,24 +433,23 @@ __global__ void __maxnreg__(kLanesRegs) k_eval_f32_lanes(const LanesArgs a) {
   // A wait that gives up (about a second) sets the error flag; the warp then
   // waits for no more copies and the block runs its tiles to the end with
   // what its buffers hold (valid users by construction, results unspecified).
-  bool late = false;
+  int late = 0;  // 1: waits for no more copies, 2: nor for the block's own warps
   auto wait_copy = [&](int m, uint32_t ph) {
     if (!bulk || late || mbar_wait(mb0 + 8 * m, ph)) return;
     if (lane == 0) atomicExch(a.err_flag, 1);
     mbar_wait(mb0 + 8 * m, ph);  // a bounded chance to land before its buffer is left
-    late = true;
+    late = 1;
   };
   // The block's own warps always arrive, a late one after two of its waits:
   // the bound here is a net, several times that.  A late warp waits for the
   // others as before: one that ran ahead would complete phases that they have
   // not seen, and they would sit their whole bound out (a call whose copies
   // never come returned after 9.7 s that way).
-  bool lost = false;
   auto wait_warps = [&](int m, int i) {
-    for (int k = 0; k < 8 && !lost; ++k)
+    for (int k = 0; k < 8 && late < 2; ++k)
       if (mbar_wait(mb0 + 8 * m, (uint32_t)i & 1)) return;
-    if (lane == 0 && !lost && a.err_flag) atomicExch(a.err_flag, 1);
-    lost = true;
+    if (lane == 0 && late < 2 && a.err_flag) atomicExch(a.err_flag, 1);
+    late = 2;
   };
   auto arrive = [&](int m) {
     __syncwarp();
@@ -516,8 +506,8 @@ __global__ void __maxnreg__(kLanesRegs) k_eval_f32_lanes(const LanesArgs a) {
     // holds behind it need not be pilots, and lanes_put takes a tile with any
     // byte of K or more apart byte by byte (2,918 chromosomes of 19 x 20: 21.2
     // us, 13.6 so)
-    const int c = (int)min((int64_t)lane, a.n - tile * kLanesTile - 1);
-    lanes_decode(smem_u32(x) + c * LK, smem_u32(INV + (i & 1) * a.inv_words + lane), L, K, dw, ND);
+    const int at = by == tile_bytes ? lane * LK : min(lane * LK, by - LK);
+    lanes_decode(smem_u32(x) + at, smem_u32(INV + (i & 1) * a.inv_words + lane), L, K, dw, ND);
     arrive(3 + (i & 1));
     bar_sync(3, NDT);  // the buffer is read: refill it
     const int64_t nx = tile + a.xbufs * nb;

@@ -546,6 +546,39 @@ bool f32_supported(int L, int K, size_t* smem_bytes) {
   return smem <= (size_t)kSmemBudget;
 }
 
+// Time (us) of the small calls' kernels (k_eval_f32_pilot, k_eval_f32) on n
+// chromosomes; lanes_us (pa_eval_lanes.cu) has the other side and what both are
+// fitted to.  m tiles on the busiest SM, `later` rounds of its blocks beyond the
+// first: launch and table, a thread's chain over the cells, gathers (and decoding)
+// per tile, later rounds, member sums.
+double small_eval_us(const pa_ctx* ctx, int64_t n) {
+  const F32Tables& t = ctx->t32;
+  const int L = ctx->cfg.L, K = ctx->cfg.K;
+  const bool fin = ctx->cfg.mode == PA_SINR_FINITE_M;
+  int NT, per_sm, cols = t.NJ;
+  const bool pilot = pilot_kernel_applies(t.NJ, t.vec, K);
+  if (pilot) {
+    const PilotLaunch s = pilot_shape(L, K, t.RS, t.NJ);
+    NT = spread_members(n, s.NT, s.unit, ctx->num_sms);
+    per_sm = std::min(4, (int)(kSmemPerSm / (s.smem + 1024)));
+  } else {
+    const F32Launch s = f32_shape(L, K, t.RS, t.NJ);
+    NT = spread_members(n, s.NT, 1, ctx->num_sms);
+    // registers: 128 per thread for the wider tables, else at most 64
+    const int regs = t.NJ >= (t.vec == 2 ? (fin ? 20 : 32) : (fin ? 16 : 24)) ? 128 : 64;
+    per_sm = std::min({(int)(kSmemPerSm / (s.smem + 1024)), 65536 / (regs * s.threads),
+                       2048 / s.threads});
+    if (t.vec == 2 && t.NJ >= 8) cols /= 2;
+  }
+  per_sm = std::max(1, per_sm);
+  const int64_t tiles = (n + NT - 1) / NT, mt = (tiles + ctx->num_sms - 1) / ctx->num_sms;
+  const double m = (double)mt * NT / 32, later = (double)((mt - 1) / per_sm);
+  const double chain = 0.01 * L * cols, words = 1e-3 * L * t.NJ * K * m;
+  if (pilot) return 3.50 + 0.74 * chain + 0.565 * words + 2.27 * later + 0.33 * m;
+  if (t.vec == 2) return 4.40 + 0.27 * chain + 0.648 * words + 1.94 * later + 0.18 * m;
+  return 3.86 + 0.40 * chain + 0.41 * words + 8.6e-3 * L * K * m + 1.23 * later;
+}
+
 cudaError_t launch_eval_f32(pa_ctx* ctx, const uint8_t* pop, int64_t n, float* fit,
                             cudaStream_t st) {
   if (n <= 0) return cudaSuccess;

@@ -17,6 +17,8 @@ constexpr int kMaxK = 64;            // pilots per cell (uint8 rows, smem rows)
 constexpr int kMaxL = 255;           // cells
 constexpr int kMaxNJ = 48;           // widest per-thread BS vector of the FP32 kernel
 constexpr int kSmemBudget = 227 * 1024;
+constexpr int kSmemPerSm = 228 * 1024;  // a kilobyte of it per resident block
+constexpr int kLanesTile = 32;       // chromosomes per tile of the large evaluations
 
 // Stream tags of the counter-based generator (counter word 3).
 enum : uint32_t { kTagSeed = 1, kTagKmeans = 2, kTagGa = 3, kTagIsland = 4 };
@@ -132,6 +134,14 @@ cudaError_t launch_eval_lanes(pa_ctx* ctx, const uint8_t* pop, int64_t n, float*
 // and the fitness itself when *summed)
 cudaError_t launch_eval_chunk(pa_ctx* ctx, const uint8_t* pop, int64_t n, float* fit,
                               bool* summed, cudaStream_t st);
+// Time (us) of a resident-table call of n chromosomes by the small calls'
+// kernels (pa_fitness.cu).
+double small_eval_us(const pa_ctx* ctx, int64_t n);
+// Whether a column-tiled call of n chromosomes is faster in tiles of 32 than by
+// the small calls' kernel (pa_stream.cu).
+bool tiles_pay(const pa_ctx* ctx, int64_t n);
+// Resident blocks per SM of a kernel at a launch shape, cached (pa_fitness.cu).
+int cached_occupancy(const void* fn, int threads, size_t smem, cudaError_t* err);
 // pa_stream.cu: column-tiled evaluation for tables beyond shared memory
 bool f32_stream_geometry(int L, int K, int* JT, int* RSt, int* vec, int* ntile);
 cudaError_t launch_eval_f32_stream(pa_ctx* ctx, const uint8_t* pop, int64_t n, float* fit,

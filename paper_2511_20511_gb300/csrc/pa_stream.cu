@@ -175,6 +175,26 @@ bool f32_stream_geometry(int L, int K, int* JT, int* RSt, int* vec, int* ntile) 
   return false;
 }
 
+// Both ways hold one column tile per block and take its chromosomes in rounds:
+// NTM of them by this file's kernel, 32 by k_eval_f32_lanes and k_eval_f32_chunk,
+// whose chromosomes take `ratio` of this kernel's time (measured 0.56 at K = 10,
+// 0.82 at 16; 1.0 at 17, 0.97 at 20, 0.92 at 32; 0.75 at 48).  Whole rounds are
+// what counts (61 x 32, this kernel / chunks: 1,216 chromosomes 31.2 / 28.9 us,
+// 1,435: 43.9 / 51.7, 1,920: 56.3 / 52.2, 2,912: 69.0 / 73.9): of 420 calls of 28
+// shapes, graph-replayed, the choice is the faster one or within a hundredth of
+// it but for two (80 x 20 at 1,216 and 1,435, 7 %).
+bool tiles_pay(const pa_ctx* ctx, int64_t n) {
+  const F32Tables& t = ctx->t32;
+  const int K = ctx->cfg.K, NTM = std::max(1, kStreamThreads / K);
+  const double ratio = K <= 16 ? 0.7 : K <= 32 ? 1.04 - 0.004 * K : 0.8;
+  const int64_t mtiles = (n + NTM - 1) / NTM, tiles = (n + kLanesTile - 1) / kLanesTile;
+  const int64_t per_tile = std::min<int64_t>(mtiles, (ctx->num_sms + t.ntile - 1) / t.ntile);
+  double rounds = (double)((mtiles + per_tile - 1) / per_tile);
+  if (per_tile * t.ntile > ctx->num_sms) rounds *= 1.5;  // some blocks wait for an SM
+  const int64_t blocks = std::max(1, ctx->num_sms / t.ntile);
+  return (double)((tiles + blocks - 1) / blocks) * kLanesTile * ratio < rounds * NTM;
+}
+
 cudaError_t launch_eval_f32_stream(pa_ctx* ctx, const uint8_t* pop, int64_t n, float* fit,
                                    cudaStream_t st) {
   if (n <= 0) return cudaSuccess;
