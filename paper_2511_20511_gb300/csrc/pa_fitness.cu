@@ -94,9 +94,16 @@ __global__ void __launch_bounds__(512) k_eval_f32(const F32Args a) {
     const int nvalid = (int)((a.n - n0) < NT ? (a.n - n0) : NT);
     decode_members(a.pop + n0 * LK, LK, nvalid, NT, L, K, INV);
     __syncthreads();
-    if (active)
-      eval_pilot_f32<NJ, VEC, FIN, JS>(sm, invp, NTK, h, PART + q * (NJ / 2) + h * (NJ / 2 / JS),
-                                       a.obj);
+    if (active) {
+      float* part = PART + q * (NJ / 2) + h * (NJ / 2 / JS);
+      // scalar rows of at most eight cells: the shorter form's registers (40, the
+      // other's 63) leave room for more blocks (7 x 40, n = 4,339: 9.6 -> 8.5 us);
+      // of more than 44 the other form spills (48 x 19, n = 55,119: 520 -> 490 us)
+      if constexpr (VEC == 1 && (NJ <= 8 || (FIN && NJ > 44)))
+        eval_pilot_short<NJ, VEC, FIN, JS>(sm, invp, NTK, h, part, a.obj);
+      else
+        eval_pilot_f32<NJ, VEC, FIN, JS>(sm, invp, NTK, h, part, a.obj);
+    }
     __syncthreads();
     for (int c = tid >> 5; c < nvalid; c += blockDim.x >> 5) {
       const float* part = PART + c * K * (NJ / 2);
