@@ -187,6 +187,14 @@ bool island_cnt_in_smem(int N, int L, int K, int C);
 size_t island_cnt_words(int L, int K, int C);
 cudaError_t launch_island_kmeans(const pa_ctx* ctx, const uint8_t* pop, int gen, int32_t* labels,
                                  cudaStream_t st);
+// pa_island_members.cu: its form for many members of few users
+cudaError_t launch_island_kmeans_mb(const pa_ctx* ctx, const uint8_t* pop, int gen, int32_t* labels,
+                                    cudaStream_t st);
+// Launch configuration of one cluster of R CTAs (attr: storage of its attribute),
+// and whether such a cluster can be resident, cached (pa_island.cu).
+cudaLaunchConfig_t cluster_config(int R, int threads, size_t smem, cudaStream_t st,
+                                  cudaLaunchAttribute* attr);
+cudaError_t cluster_resident(const void* fn, int dev, const cudaLaunchConfig_t& cfg, bool* ok);
 cudaError_t launch_island_lists(const pa_ctx* ctx, const int32_t* labels, const IslandLists& il,
                                 cudaStream_t st);
 cudaError_t launch_island_step(const pa_ctx* ctx, const uint8_t* pop, const void* fit,

@@ -21,8 +21,10 @@
 // changes or the pass limit; an emptied cluster keeps its counts.
 // k_island_kmeans_cl runs it on a cluster of up to sixteen CTAs when their
 // shares of counts and population fit in shared memory (the users are split
-// over the CTAs); k_island_kmeans on one CTA otherwise (counts in global
-// memory for large C*L*K*K, rows read from global memory for large N*L*K).
+// over the CTAs); k_island_kmeans_mb (pa_island_members.cu) on a cluster of up to
+// eight with the members split, for many members of few users; k_island_kmeans on
+// one CTA otherwise (counts in global memory for large C*L*K*K, rows read from
+// global memory for large N*L*K).
 
 // Island lists (k_island_lists): members grouped by island in ascending
 // index (off, list) and each member's position in its island (pos), by a
@@ -562,67 +564,80 @@ size_t island_cnt_words(int L, int K, int C) {
   return (size_t)L * K * K * (((C + 1) / 2) | 1);
 }
 
-// Cluster form of the K-means (k_island_kmeans_cl): the largest of 16, 8, 4
-// or 2 CTAs that can be resident, with 16 members and (above 2 CTAs) a word of
-// four users for each; where none of those fits, CTAs without users too.
-// cudaErrorNotSupported when it does not apply (fewer than 64 members, a
-// layout beyond shared memory, no cluster shape resident).
-cudaError_t launch_island_kmeans_cl(const pa_ctx* ctx, const uint8_t* pop, int gen, int32_t* labels,
-                                    cudaStream_t st) {
-  const pa_config& c = ctx->cfg;
-  if (c.N < 64) return cudaErrorNotSupported;
-  // residency of a shape, once per (device, cluster size, shared memory)
+cudaLaunchConfig_t cluster_config(int R, int threads, size_t smem, cudaStream_t st,
+                                  cudaLaunchAttribute* attr) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(R, 1, 1);
+  cfg.blockDim = dim3(threads, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  attr->id = cudaLaunchAttributeClusterDimension;
+  attr->val.clusterDim.x = R;
+  attr->val.clusterDim.y = 1;
+  attr->val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cfg;
+}
+
+// The first query of a kernel on a device raises its shared-memory cap and allows
+// clusters above the portable size.
+cudaError_t cluster_resident(const void* fn, int dev, const cudaLaunchConfig_t& cfg, bool* ok) {
   struct Fit {
-    int dev, R, smem;
+    const void* fn;
+    int dev, R;
+    size_t smem;
     bool ok;
   };
   static std::vector<Fit> fits;
   static std::mutex mu;
-  static std::atomic<uint64_t> capped{0};
-  const uint64_t bit = 1ULL << (ctx->device & 63);
-  if (!(capped.load() & bit)) {
-    cudaError_t e = raise_smem_cap((const void*)k_island_kmeans_cl, ctx->device);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(k_island_kmeans_cl, cudaFuncAttributeNonPortableClusterSizeAllowed,
-                               1);
-    if (e != cudaSuccess) return e;
-    capped.fetch_or(bit);
+  std::lock_guard<std::mutex> lock(mu);
+  const int R = (int)cfg.gridDim.x;
+  bool seen = false;
+  for (const Fit& f : fits) {
+    if (f.fn != fn || f.dev != dev) continue;
+    seen = true;
+    if (f.R == R && f.smem == cfg.dynamicSmemBytes) {
+      *ok = f.ok;
+      return cudaSuccess;
+    }
   }
-  const int W = (c.L * c.K + 3) / 4;
+  if (!seen) {
+    cudaError_t e = raise_smem_cap(fn, dev);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+  }
+  int nclusters = 0;
+  *ok = cudaOccupancyMaxActiveClusters(&nclusters, fn, &cfg) == cudaSuccess && nclusters >= 1;
+  (void)cudaGetLastError();
+  if (fits.size() < 256) fits.push_back(Fit{fn, dev, R, cfg.dynamicSmemBytes, *ok});
+  return cudaSuccess;
+}
+
+// Cluster form of the K-means (k_island_kmeans_cl): the largest of 16, 8, 4
+// or 2 CTAs that can be resident, with 16 members and (above 2 CTAs) a word of
+// four users for each; where none of those fits, CTAs without users too.
+// cudaErrorNotSupported when it does not apply (fewer than 64 members, a
+// layout beyond shared memory, or with room for the sums only in more than 16
+// pieces, a cluster barrier each: 7 x 10, N = 4000, C = 64 343 us per pass, 258 on one
+// CTA; no cluster shape resident).
+cudaError_t launch_island_kmeans_cl(const pa_ctx* ctx, const uint8_t* pop, int gen, int32_t* labels,
+                                    cudaStream_t st) {
+  const pa_config& c = ctx->cfg;
+  if (c.N < 64) return cudaErrorNotSupported;
+  const int W = (c.L * c.K + 3) / 4, CW = (c.islands + 1) / 2;
   for (int t = 0; t < 8; ++t) {
     const int R = 16 >> (t & 3);
     if ((R > 2 && R > W) != (t >= 4) || 16 * R > c.N) continue;
     const KmClLayout k = km_cl_layout(c.N, c.L, c.K, c.islands, R, kKmClThreads,
                                       (int)kKmSmemBudget);
-    if ((size_t)k.total > kKmSmemBudget) continue;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(R, 1, 1);
-    cfg.blockDim = dim3(kKmClThreads, 1, 1);
-    cfg.dynamicSmemBytes = k.total;
-    cfg.stream = st;
+    if ((size_t)k.total > kKmSmemBudget || CW > 16 * k.CWc) continue;
     cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = R;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    const cudaLaunchConfig_t cfg = cluster_config(R, kKmClThreads, k.total, st, attr);
     bool ok = false;
-    {
-      std::lock_guard<std::mutex> lock(mu);
-      auto it = std::find_if(fits.begin(), fits.end(), [&](const Fit& f) {
-        return f.dev == ctx->device && f.R == R && f.smem == k.total;
-      });
-      if (it == fits.end()) {
-        int nclusters = 0;
-        ok = cudaOccupancyMaxActiveClusters(&nclusters, k_island_kmeans_cl, &cfg) ==
-                 cudaSuccess && nclusters >= 1;
-        (void)cudaGetLastError();
-        if (fits.size() < 256) fits.push_back(Fit{ctx->device, R, k.total, ok});
-      } else {
-        ok = it->ok;
-      }
-    }
+    cudaError_t e = cluster_resident((const void*)k_island_kmeans_cl, ctx->device, cfg, &ok);
+    if (e != cudaSuccess) return e;
     if (!ok) continue;
     KmClArgs a;
     a.pop = pop;
@@ -631,7 +646,7 @@ cudaError_t launch_island_kmeans_cl(const pa_ctx* ctx, const uint8_t* pop, int g
     a.label = labels;
     a.passes = ctx->isl_passes;
     (void)cudaGetLastError();  // drop a stale error of an earlier call
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_island_kmeans_cl, a);
+    e = cudaLaunchKernelEx(&cfg, k_island_kmeans_cl, a);
     count_launch();
     return e;
   }
@@ -641,8 +656,9 @@ cudaError_t launch_island_kmeans_cl(const pa_ctx* ctx, const uint8_t* pop, int g
 cudaError_t launch_island_kmeans(const pa_ctx* ctx, const uint8_t* pop, int gen, int32_t* labels,
                                  cudaStream_t st) {
   const pa_config& c = ctx->cfg;
-  {  // the cluster form, where it fits and can be resident
-    cudaError_t e = launch_island_kmeans_cl(ctx, pop, gen, labels, st);
+  {  // a cluster form, where one fits and can be resident
+    cudaError_t e = launch_island_kmeans_mb(ctx, pop, gen, labels, st);
+    if (e == cudaErrorNotSupported) e = launch_island_kmeans_cl(ctx, pop, gen, labels, st);
     if (e != cudaErrorNotSupported) return e;
   }
   const bool cs = ctx->isl_cnt == nullptr;
