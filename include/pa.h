@@ -175,7 +175,11 @@ pa_status pa_set_stream(pa_ctx* ctx, void* stream);
  * in shared memory with bulk copies under a bounded wait (about a second);
  * a wait that gives up leaves the outputs unspecified and is reported as
  * PA_ETIMEOUT by the context's next synchronous call
- * (pa_eval_population_host, pa_solve, pa_get_population).
+ * (pa_eval_population_host, pa_solve, pa_get_population).  Device memory:
+ * where the FP32 table exceeds one SM's shared memory (61 cells x 32 users),
+ * the first call of a size makes the context keep 4 bytes per chromosome and
+ * column tile, and with K > 16 also decoded chromosomes, at most 256 MB (a
+ * call runs without them when they cannot be had), until pa_destroy.
  */
 pa_status pa_eval_population(pa_ctx* ctx, const uint8_t* pop_dev, int64_t n, void* fit_dev);
 

@@ -37,7 +37,9 @@ constexpr int kChunkCells = 8;
 constexpr int kChunkBufs = 4;
 constexpr int kChunkThreads = 1024;
 constexpr int kDecodeThreads = 256;
-constexpr int64_t kChunkSlab = 1 << 17;  // chromosomes whose inverses are held at once
+// chromosomes whose inverses are held at once, and their bytes, at most
+constexpr int64_t kChunkSlab = 1 << 17;
+constexpr int64_t kChunkBytes = 256 << 20;
 
 // Words of one chunk of one tile's inverse, and chunks per tile.
 __host__ __device__ constexpr int chunk_words(int K) { return kChunkCells / 4 * K * kLanesTile; }
@@ -377,8 +379,8 @@ cudaError_t run_chunk(const LanesArgs& a, const F32Tables& t, float* fit, int* t
 // Column-tiled tables with K > 16 (scalar rows): the fitness of n chromosomes;
 // t.partial holds n * ntile values.  cudaErrorNotSupported for other tables,
 // small calls (tiles_pay), or where it does not fit (shared memory, or
-// device memory for the inverses of kChunkSlab chromosomes: the context keeps
-// them, at most 256 MB or so).  *summed: fit is written, else the caller adds
+// device memory for the inverses of a slab of chromosomes: the context keeps
+// them, at most kChunkBytes).  *summed: fit is written, else the caller adds
 // the partials.  Where a block has few tiles, tickets save the launch that adds
 // the partials (4 us of a generation's 78 at n = 2048, all launches ordinary); with many, the fence
 // behind each tile costs more (2^17: 2,428 us against 2,348).
@@ -410,13 +412,15 @@ cudaError_t launch_eval_chunk(pa_ctx* ctx, const uint8_t* pop, int64_t n, float*
   a.o_x = (int)b;
   b += 4 * (size_t)a.EW * PPW * (t.JT / 4) * kLanesTile;
   if (b + 1024 > (size_t)kSmemBudget) return cudaErrorNotSupported;
-  const int64_t slab = std::min(n, kChunkSlab), slab_tiles = (slab + kLanesTile - 1) / kLanesTile;
   const int nch = chunk_count(L);
+  const int64_t tile_bytes = 4 * (int64_t)a.inv_words * nch;
+  const int64_t slab = std::min({n, kChunkSlab, kChunkBytes / tile_bytes * kLanesTile});
+  const int64_t slab_tiles = (slab + kLanesTile - 1) / kLanesTile;
   if (t.inv_cap < slab_tiles) {
     cudaFree(t.inv);
     t.inv = nullptr;
     t.inv_cap = 0;
-    const size_t inv_bytes = 4 * (size_t)a.inv_words * nch * slab_tiles;
+    const size_t inv_bytes = (size_t)(tile_bytes * slab_tiles);
     if (cudaMalloc(&t.inv, inv_bytes + sizeof(int) * slab_tiles) != cudaSuccess) {
       (void)cudaGetLastError();
       return cudaErrorNotSupported;
@@ -436,7 +440,7 @@ cudaError_t launch_eval_chunk(pa_ctx* ctx, const uint8_t* pop, int64_t n, float*
   a.pc = t.pc;
   a.obj = ctx->cfg.objective;
   const bool fin = ctx->cfg.mode == PA_SINR_FINITE_M;
-  *summed = slab_tiles * t.ntile <= 4 * (int64_t)ctx->num_sms;  // (then one slab)
+  *summed = n <= slab && slab_tiles * t.ntile <= 4 * (int64_t)ctx->num_sms;
   int* tickets = *summed ? t.tickets : nullptr;
   for (int64_t n0 = 0; n0 < n; n0 += slab) {
     a.n = std::min(slab, n - n0);
