@@ -417,12 +417,19 @@ cudaError_t launch_eval_chunk(pa_ctx* ctx, const uint8_t* pop, int64_t n, float*
   const int64_t slab = std::min({n, kChunkSlab, kChunkBytes / tile_bytes * kLanesTile});
   const int64_t slab_tiles = (slab + kLanesTile - 1) / kLanesTile;
   if (t.inv_cap < slab_tiles) {
+    // not while the stream is captured (an allocation would end the capture), nor
+    // again where it failed
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) (void)cudaGetLastError();
+    if (cap != cudaStreamCaptureStatusNone || t.inv_none <= slab_tiles)
+      return cudaErrorNotSupported;
     cudaFree(t.inv);
     t.inv = nullptr;
     t.inv_cap = 0;
     const size_t inv_bytes = (size_t)(tile_bytes * slab_tiles);
     if (cudaMalloc(&t.inv, inv_bytes + sizeof(int) * slab_tiles) != cudaSuccess) {
       (void)cudaGetLastError();
+      t.inv_none = slab_tiles;
       return cudaErrorNotSupported;
     }
     t.tickets = reinterpret_cast<int*>(reinterpret_cast<unsigned char*>(t.inv) + inv_bytes);

@@ -49,6 +49,7 @@ struct F32Tables {
   int64_t partial_cap = 0;   // members it can hold
   uint32_t* inv = nullptr;   // scratch: decoded inverses (pa_eval_chunk.cu)
   int64_t inv_cap = 0;       // tiles of 32 members it can hold
+  int64_t inv_none = INT64_MAX;  // tiles it could not be allocated for
   int* tickets = nullptr;    // one per such tile, behind inv; zero between launches
   int* err_flag = nullptr;   // set by a kernel whose bounded wait gave up
 };

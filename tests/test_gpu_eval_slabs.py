@@ -60,3 +60,47 @@ def test_several_slabs(B, L, K, ntile):
             assert torch.equal(_eval(B, ctx, pop[a:b].contiguous()), fit[a:b])
     finally:
         B.pa_destroy(ctx)
+
+
+def test_no_memory_for_the_inverses(B):
+    """Where the inverses cannot be had the call takes a kernel that needs none,
+    again and again, also while its stream is being captured."""
+    L, K, n = 61, 32, 1 << 16
+    st = torch.cuda.Stream()
+    with torch.cuda.stream(st):
+        cfg = B.pa_config_default(L, K, mode=1, M=256.0, rho=1e9, N=32)
+        beta = _beta(L, K)
+        plain, ctx = B.pa_create(cfg, beta, stream=st), B.pa_create(cfg, beta, stream=st)
+        hold = None
+        try:
+            pop = inputs.random_population_torch(n, L, K, 3, "cuda")
+            fit = torch.empty(n, dtype=torch.float32, device="cuda")
+            B.pa_eval_population(plain, pop, fit)
+            want = fit.clone()
+            B.pa_eval_population(ctx, pop[:64], fit[:64])  # its kernel is loaded
+            warm = torch.cuda.CUDAGraph()
+            st.synchronize()
+            with torch.cuda.graph(warm, stream=st):
+                B.pa_eval_population(ctx, pop[:64], fit[:64])
+            st.synchronize()
+            torch.cuda.empty_cache()
+            # 128 MB and a little would be needed
+            hold = torch.empty(torch.cuda.mem_get_info()[0] - (100 << 20), dtype=torch.uint8,
+                               device="cuda")
+            for _ in range(2):
+                fit.fill_(-1.0)
+                B.pa_eval_population(ctx, pop, fit)
+                assert torch.equal(fit, want)
+            st.synchronize()
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph, stream=st):
+                B.pa_eval_population(ctx, pop, fit)
+            fit.fill_(-1.0)
+            graph.replay()
+            assert torch.equal(fit, want)
+        finally:
+            del hold
+            st.synchronize()
+            B.pa_destroy(ctx)
+            B.pa_destroy(plain)
+            torch.cuda.empty_cache()
