@@ -34,9 +34,9 @@
 // products (no FMA), log2 by the atanh series, per-cell partial sums added in
 // ascending j.
 #include <algorithm>
-#include <mutex>
 
 #include "pa_eval_device.cuh"
+#include "pa_occ_cache.cuh"
 
 namespace pa {
 namespace {
@@ -387,49 +387,18 @@ F32Launch f32_shape(int L, int K, int RS, int NJ) {
 // Resident blocks per SM of a kernel at a launch shape.  The first query of
 // a kernel on a device raises its dynamic shared-memory cap to the device's
 // opt-in maximum (a cap sized to one launch would reject a later, larger
-// one); the queries cost host time, so results are cached per (kernel,
-// device, threads, shared memory).
-struct OccKey {
-  const void* fn;
-  int dev, threads;
-  size_t smem;
-};
+// one); the queries cost host time, so results are cached.
 int cached_occupancy(const void* fn, int threads, size_t smem, cudaError_t* err) {
-  static OccKey keys[256];
-  static int vals[256];
-  static int used = 0;
-  static const void* capped_fn[64];
-  static int capped_dev[64];
-  static int ncapped = 0;
-  static std::mutex mu;
-  std::lock_guard<std::mutex> lock(mu);
-  int dev = 0;
+  static OccCache cache;
+  int dev = 0, per_sm = 0;
   *err = cudaGetDevice(&dev);
   if (*err != cudaSuccess) return 0;
-  for (int i = 0; i < used; ++i)
-    if (keys[i].fn == fn && keys[i].dev == dev && keys[i].threads == threads &&
-        keys[i].smem == smem)
-      return vals[i];
-  bool capped = false;
-  for (int i = 0; i < ncapped; ++i) capped |= (capped_fn[i] == fn && capped_dev[i] == dev);
-  if (!capped) {
-    *err = raise_smem_cap(fn, dev);
-    if (*err != cudaSuccess) return 0;
-    if (ncapped < 64) {
-      capped_fn[ncapped] = fn;
-      capped_dev[ncapped] = dev;
-      ++ncapped;
-    }
-  }
-  int per_sm = 0;
-  *err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem);
-  if (*err != cudaSuccess) return 0;
-  if (used < 256) {
-    keys[used] = OccKey{fn, dev, threads, smem};
-    vals[used] = per_sm;
-    ++used;
-  }
-  return per_sm;
+  *err = (cudaError_t)cache.get(
+      OccKey{fn, dev, threads, smem}, &per_sm, [&] { return (int)raise_smem_cap(fn, dev); },
+      [&](int* v) {
+        return (int)cudaOccupancyMaxActiveBlocksPerMultiprocessor(v, fn, threads, smem);
+      });
+  return *err == cudaSuccess ? per_sm : 0;
 }
 
 namespace {
