@@ -72,14 +72,6 @@ struct SolveArgs {
   int32_t* isl_pos_out;
 };
 
-template <typename FT>
-__device__ __forceinline__ bool better_s(const FT* fit, int a, int b) {
-  const FT fa = fit[a], fb = fit[b];
-  if (fa > fb) return true;
-  if (fa < fb) return false;
-  return a < b;
-}
-
 // "member i with fitness v is better than member b with fitness bv": higher
 // fitness, or not lower (equal or unordered) and a lower index.
 template <typename FT>
@@ -235,87 +227,6 @@ __device__ __forceinline__ int warp_rank_list(const FT* fit, const int* mem, int
   return last;
 }
 
-// The member of rank i (fitness desc, index asc) among the m members
-// mem[0..m), i < min(m, kSmallE), by the sixteen lanes of `mask` (a half-warp)
-// in i + 1 rounds of an argmax.  Each of them gets it.
-template <typename FT>
-__device__ __forceinline__ int half_rank_list(const FT* fit, const int* mem, int m, int i,
-                                              unsigned mask, int hl) {
-  int chosen[kSmallE], last = -1;
-#pragma unroll
-  for (int e = 0; e < kSmallE; ++e) {
-    chosen[e] = -1;
-    if (e <= i) {
-      int best = -1;
-      FT bv = (FT)0;
-      for (int t = hl; t < m; t += 16) {
-        const int c = mem[t];
-        bool taken = false;
-#pragma unroll
-        for (int f = 0; f < e; ++f) taken |= chosen[f] == c;
-        if (taken) continue;
-        const FT v = fit[c];
-        if (best < 0 || better_v(v, c, bv, best)) {
-          best = c;
-          bv = v;
-        }
-      }
-#pragma unroll
-      for (int off = 8; off > 0; off >>= 1) {
-        const int o = __shfl_xor_sync(mask, best, off);
-        const FT ov = __shfl_xor_sync(mask, bv, off);
-        if (o >= 0 && (best < 0 || better_v(ov, o, bv, best))) {
-          best = o;
-          bv = ov;
-        }
-      }
-      chosen[e] = last = best;
-    }
-  }
-  return last;
-}
-
-// Block-wide best member by (fitness desc, index asc), skipping excluded[0..nex).
-template <typename FT>
-__device__ int block_best_s(const FT* fit, int N, const int* excluded, int nex, int* red) {
-  int best = -1;
-  for (int i = threadIdx.x; i < N; i += blockDim.x) {
-    bool skip = false;
-    for (int e = 0; e < nex; ++e) skip |= (excluded[e] == i);
-    if (skip) continue;
-    if (best < 0 || better_s(fit, i, best)) best = i;
-  }
-  for (int off = 16; off > 0; off >>= 1) {
-    const int o = __shfl_down_sync(0xffffffffu, best, off);
-    if (o >= 0 && (best < 0 || better_s(fit, o, best))) best = o;
-  }
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = best;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int b = -1;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-      const int o = red[w];
-      if (o >= 0 && (b < 0 || better_s(fit, o, b))) b = o;
-    }
-    red[32] = b;
-  }
-  __syncthreads();
-  const int r = red[32];
-  __syncthreads();
-  return r;
-}
-
-__device__ __forceinline__ void swap2(uint8_t* row, int K, uint32_t ui, uint32_t uj) {
-  if (K < 2) return;
-  const int i = (int)below(ui, (uint32_t)K);
-  const int jj = (int)below(uj, (uint32_t)(K - 1));
-  const int j = jj + (jj >= i ? 1 : 0);
-  const uint8_t t = row[i];
-  row[i] = row[j];
-  row[j] = t;
-}
-
 // A child's 32-bit word from its parents' words: the first na bytes from
 // parent A, the rest from parent B (na <= 0: all B; na >= 4: all A) -- the
 // word holding a row-wise crossover cut.
@@ -447,6 +358,7 @@ __device__ __forceinline__ void solve_body(const SolveArgs& a, unsigned char* sm
   constexpr int NPR = NJ / 2;  // column pairs per (member, pilot)
   // the batched column split (many members per CTA) may build two children per warp
   constexpr bool kHalves = MAXNP != kSoloMaxNP;
+  static_assert(!(ISL && kHalves), "islands run on the one-instance column split");
 
   // ---- carve shared memory
   unsigned char* p = smem;
@@ -817,33 +729,18 @@ __device__ __forceinline__ void solve_body(const SolveArgs& a, unsigned char* sm
           const int n = base_n + slot;
           const uint32_t* dr = DR + (size_t)i * nblk * 8;
           uint32_t* child = reinterpret_cast<uint32_t*>(popn + slot * MS);
-          // Candidates: all members, or the island's.  Slot n of island c at
-          // position i is the island's rank-i member for i < min(E, m_c), found
-          // by this slot's lanes while the others build their children (a search
-          // of all islands before the children took 1.8 us of a 256-member
-          // generation's 7.3), else a child of two tournaments in the island.
-          const int* mem = nullptr;
-          int m = N, irank = -1;
-          bool elite = !isl && n < E;
-          if (isl) {
-            const int c = ilab[n], at = ipos[n];
-            mem = ilist + ioff[c];
-            m = ioff[c + 1] - ioff[c];
-            elite = at < min(E, m);
-            irank = at;
-          }
+          const bool elite = n < E;
           int pa_, pb_;
           int split = LK;
           if (elite) {
-            pa_ = pb_ = isl ? half_rank_list<FT>(fit, mem, m, irank, hmask, hl) : elites[n];
+            pa_ = pb_ = elites[n];
           } else {
             if (T_ <= 8) {  // eight lanes a tournament, a candidate each
               const int t = lane & 7;
               int c = -1;
               FT v = (FT)0;
               if (t < T_) {
-                c = (int)below(dr[((lane >> 3) & 1) * T_ + t], (uint32_t)m);
-                if (isl) c = mem[c];
+                c = (int)below(dr[((lane >> 3) & 1) * T_ + t], (uint32_t)N);
                 v = fit[c];
               }
               for (int off = T_ > 4 ? 4 : 2; off > 0; off >>= 1) {
@@ -856,9 +753,6 @@ __device__ __forceinline__ void solve_body(const SolveArgs& a, unsigned char* sm
               }
               pa_ = __shfl_sync(hmask, c, lane & 16);
               pb_ = __shfl_sync(hmask, c, (lane & 16) + 8);
-            } else if (isl) {
-              pa_ = tournament_list(fit, mem, m, T_, dr);
-              pb_ = tournament_list(fit, mem, m, T_, dr + T_);
             } else {
               pa_ = tournament_lane(fit, N, T_, dr);
               pb_ = tournament_lane(fit, N, T_, dr + T_);
@@ -872,7 +766,7 @@ __device__ __forceinline__ void solve_body(const SolveArgs& a, unsigned char* sm
           const int ob = nt_shift >= 0 ? pb_ >> nt_shift : pb_ / NT;
           const uint32_t ra = dsmem_addr(POPp(cur) + (pa_ - oa * NT) * MS, oa);
           const uint32_t rb = dsmem_addr(POPp(cur) + (pb_ - ob * NT) * MS, ob);
-  #pragma unroll 2
+#pragma unroll 2
           for (int v = hl; v < (MS >> 4); v += 16) {
             const uint4 qa = ld_dsmem_v4(ra + 16 * v), qb = ld_dsmem_v4(rb + 16 * v);
             // bytes below sp from A: the cut in X, and the same cut in INV
