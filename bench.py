@@ -46,7 +46,7 @@ BATCH_LOG2 = 20
 # DRAM bytes (read + write) per launch of the two roofline kernels, from one
 # ncu capture of each; None while a kernel has changed since its capture
 TRAFFIC_K_SOLVE = 146_688
-TRAFFIC_EVAL = 204_793_856
+TRAFFIC_EVAL = 204_561_152
 METRIC = ("chromosome fitness evals/sec and GA gens/sec (L=19,K=10); "
           "p50/p99 solve latency served vs plain")
 WORKLOAD = ("single instance at paper-like scale: L=19 hex cells (2 rings), K=10 users/cell, "

@@ -24,19 +24,19 @@
 //     which share the data path).
 // A unit holds at most six column pairs, so that 36 warps of 56 registers fit
 // an SM, and keeps its code short (with decoding in every warp's path the
-// instruction cache missed: 720 us against 576 below).  Rows and own gains are
-// addressed by one dp4a each, columns are processed as f32x2 pairs (637 -> 440
+// instruction cache missed: 720 us against 571 below).  Rows and own gains are
+// addressed by one dp4a each, columns are processed as f32x2 pairs (637 -> 406
 // warp instructions per chromosome).
 // Helper warps decode tile i+1 and sum tile i-1 while the evaluation warps
 // gather tile i, so the data path stays busy through those phases; warps wait
 // for one another only through mbarriers (a tile of slack), not through block
 // barriers.  Chromosome bytes arrive by one bulk copy per tile, the table by
 // bulk copies at the start.
-// Measured (GB300, finite-M SINR): 2^20 chromosomes of 19 x 10 in 576 us, 6,570
-// Gword/s of gathers, the data path 82-84 % busy with 147 wavefronts per
-// chromosome (the kernel with a thread per (chromosome, pilot): 739 us, 177
-// wavefronts); 65,536 of 37 x 16 in 201 us (370 us); of 19 x 24 in 102 us
-// (149 us); of 61 x 12, column tiles, in 453 us (618 us).
+// Measured (GB300, finite-M SINR): 2^20 chromosomes of 19 x 10 in 571 us, 6,630
+// Gword/s of gathers, the data path 85 % busy with 145 wavefronts per chromosome
+// (the kernel with a thread per (chromosome, pilot): 739 us, 177 wavefronts);
+// 65,536 of 37 x 16 in 194 us (370 us); 100,003 of 19 x 24 in 141 us (224 us); 65,536
+// of 61 x 12, column tiles, in 408 us (618 us).
 #pragma once
 
 #include <algorithm>
@@ -505,7 +505,7 @@ __global__ void __maxnreg__(kLanesRegs) k_eval_f32_lanes(const LanesArgs a) {
     // lanes past the last chromosome decode that one again: what the buffer
     // holds behind it need not be pilots, and lanes_put takes a tile with any
     // byte of K or more apart byte by byte (2,918 chromosomes of 19 x 20: 21.2
-    // us, 13.6 so)
+    // us, 14.6 so)
     const int at = by == tile_bytes ? lane * LK : min(lane * LK, by - LK);
     lanes_decode(smem_u32(x) + at, smem_u32(INV + (i & 1) * a.inv_words + lane), L, K, dw, ND);
     arrive(3 + (i & 1));

@@ -444,11 +444,11 @@ PilotLaunch pilot_shape(int L, int K, int RS, int NJ) {
 // blocks take, what spreads them over the SMs (a multiple of unit); the block
 // keeps its threads and shared memory.  A block of few members has its chain of
 // decode, gathers and sums shorter by the data path's share.
-// Per call, back to back, full blocks / spread (and the pilot kernel's chromosome
-// copies issued before the table's staging instead of behind it):
-//   19 x 10  n = 256: 10.2 / 8.2 us   2048: 10.3 / 8.2
-//   37 x 13  n = 256: 12.3 / 8.2 us   1024: 12.3 / 10.4
-//   19 x 24  n = 256: 10.3 / 8.2 us   16 x 16  n = 32: 8.2 / 6.2
+// Per call in a replayed graph, full blocks / spread (and the pilot kernel's
+// chromosome copies issued before the table's staging instead of behind it):
+//   19 x 10  n = 100: 7.6 / 6.4 us   2432: 7.8 / 7.1
+//   37 x 13  n = 100: 10.5 / 7.1 us  1216: 10.8 / 9.6
+//   19 x 24  n = 467: 8.1 / 6.2 us   16 x 16  n = 467: 6.2 / 5.3
 int spread_members(int64_t n, int NT, int unit, int num_sms) {
   const int64_t per = (n + num_sms - 1) / num_sms;
   return (int)std::min<int64_t>(NT, std::max<int64_t>(1, (per + unit - 1) / unit) * unit);

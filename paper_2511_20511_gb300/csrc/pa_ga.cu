@@ -228,10 +228,11 @@ __device__ __forceinline__ void ga_copy(uint8_t* child, const uint8_t* A, const 
 // copied into shared memory in units of up to 16 bytes, the per-row swaps there
 // (a lane a row), and the child written out.  The last block finds the elites
 // meanwhile.  What bounds it is latency: a chain of one Philox block, a fitness
-// load, a parent load and the stores (61 x 32, N = 2048, cold caches: 17 us; with
-// a block per eight children, the elites searched by the first of them before
-// its children, tournaments re-reading the fitness at each comparison and rows
-// copied bytewise: 25.4 us).  Launched early: a block may start while the
+// load, a parent load and the stores (61 x 32, N = 2048: 10.5 us with cold caches,
+// 5.8 us a call in a replayed graph; with a block per eight children, the elites
+// searched by the first of them before its children, tournaments re-reading the
+// fitness at each comparison and rows copied bytewise: 25.4 and 18.6 us).  Launched
+// early: a block may start while the
 // evaluation's last blocks run, and has its first children's draws by the time
 // the fitness is there.
 template <typename FT>
