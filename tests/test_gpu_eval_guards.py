@@ -2,9 +2,9 @@
 rows that are no permutations (pilots >= K, repeated pilots) leave every other
 chromosome's fitness as it was, and copies that never arrive end in
 PA_ETIMEOUT within seconds, after which the same context evaluates as before.
-The counts are a multiple of the SM count far above the lines at which these
-kernels take over (at most ten tiles of 32 per SM), so that a redrawn line does
-not move a case to another kernel."""
+The counts are a multiple of the SM count far above those at which these
+kernels take over (by estimated times, from one to ten tiles of 32 per SM), so that
+other estimates do not move a case to another kernel."""
 import time
 
 import numpy as np
@@ -40,7 +40,7 @@ def _beta(L, K):
 
 def _count(L, K):
     sms = torch.cuda.get_device_properties(0).multi_processor_count
-    return (16 if L <= 37 else 2) * 32 * sms + 5  # a ragged last tile
+    return (64 if L <= 37 else 2) * 32 * sms + 5  # a ragged last tile
 
 
 def _eval(B, ctx, pop):
